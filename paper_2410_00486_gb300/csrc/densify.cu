@@ -5,10 +5,10 @@
 // k_densify_plan classifies every Gaussian in float32 (0 prune, 1 keep, 2 keep + clone,
 // 3 split into two) from its average view-space gradient accum/denom, its largest
 // log-scale and its opacity logit, against thresholds rounded once from double on the
-// host; k_count_scan turns the per-Gaussian output counts into output positions and the
-// new Gaussian count; k_densify_apply writes the new parameter vector and Adam state
-// (clones and split children start with zero moments), each Gaussian's outputs
-// consecutive.  Split children are mean + R(q) (s * z) with caller-supplied standard
+// host, and sums the outputs of its span of Gaussians; k_span_scan turns the codes into
+// output positions and the new Gaussian count; k_densify_apply writes the new parameter
+// vector and Adam state (clones and split children start with zero moments), each Gaussian's
+// outputs consecutive.  Split children are mean + R(q) (s * z) with caller-supplied standard
 // normal z, scale s / 1.6, other attributes copied.
 #include <math.h>
 #include <stdio.h>
@@ -19,11 +19,114 @@ namespace cgs {
 
 constexpr float kLogSplitDiv = 0.47000362924573558f;   // ln(1.6)
 
-__global__ void k_densify_plan(const float *__restrict__ P, int64_t n, const float *__restrict__ accum,
-                               const float *__restrict__ denom, float t_grad, float t_logs, float t_logit,
-                               uint32_t *__restrict__ code, uint32_t *__restrict__ count)
+// Exclusive scan of count[0..n) into off[0..n], off[n] = total, in two launches over at most
+// kScanBlocks spans of scan_span(n) entries: the totals of the spans (formed by whichever
+// kernel has the counts at hand), then every block adds the totals before its own and scans
+// its span, 4 entries a thread.  One block walking all entries, 32 lanes of each warp at a
+// time, left the chip idle for the latency of thousands of dependent steps (200k entries 79
+// us, two launches now 3.6 us with the totals formed by the plan; 357k cells 135 -> 7 us).
+constexpr int kScanThreads = 256, kScanChunk = 4 * kScanThreads, kScanBlocks = 1024;
+
+inline int64_t scan_span(int64_t n)
 {
-    for (int64_t g = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; g < n; g += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t per = (n + kScanBlocks - 1) / kScanBlocks;
+    return (per + kScanChunk - 1) / kScanChunk * kScanChunk;
+}
+inline int scan_blocks(int64_t n) { return (int)((n + scan_span(n) - 1) / scan_span(n)); }
+
+// Sum of x over the block, returned to every thread.
+__device__ __forceinline__ unsigned long long block_sum(unsigned long long x)
+{
+    __shared__ unsigned long long ws[32];
+    for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(kFull, x, o);
+    __syncthreads();   // the previous sum has been read
+    if ((threadIdx.x & 31) == 0) ws[threadIdx.x >> 5] = x;
+    __syncthreads();
+    unsigned long long t = 0;
+    for (int i = 0; i < (int)(blockDim.x >> 5); i++) t += ws[i];
+    return t;
+}
+
+__global__ void __launch_bounds__(kScanThreads)
+k_span_totals(const uint32_t *__restrict__ count, int64_t n, int64_t span, unsigned long long *__restrict__ part)
+{
+    const int64_t lo = blockIdx.x * span, hi = min(n, lo + span);
+    unsigned long long s = 0;
+#pragma unroll 4
+    for (int64_t t = lo + threadIdx.x; t < hi; t += kScanThreads) s += count[t];
+    s = block_sum(s);
+    if (threadIdx.x == 0) part[blockIdx.x] = s;
+}
+
+// Entries of a scan: a count array, or densification codes (a pruned Gaussian leaves no
+// output, a kept one one, a cloned or split one two).
+struct CountEntry {
+    const uint32_t *count;
+    __device__ __forceinline__ uint32_t operator()(int64_t i) const { return count[i]; }
+};
+struct CodeEntry {
+    const uint32_t *code;
+    __device__ __forceinline__ uint32_t operator()(int64_t i) const { return min(code[i], 2u); }
+};
+
+template <class Entry>
+__global__ void __launch_bounds__(kScanThreads)
+k_span_scan(Entry entry, int64_t n, int64_t span, const unsigned long long *__restrict__ part,
+            uint32_t *__restrict__ off, int64_t *__restrict__ total_out)
+{
+    __shared__ uint32_t wtot[kScanThreads / 32];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    unsigned long long before = 0;
+    for (int b = threadIdx.x; b < (int)blockIdx.x; b += kScanThreads) before += part[b];
+    unsigned long long run = block_sum(before);
+    const int64_t lo = blockIdx.x * span, hi = min(n, lo + span);
+    for (int64_t base = lo; base < hi; base += kScanChunk) {
+        const int64_t t0 = base + 4 * (int64_t)threadIdx.x;
+        uint32_t c[4], tot = 0;
+#pragma unroll
+        for (int k = 0; k < 4; k++) {
+            c[k] = t0 + k < hi ? entry(t0 + k) : 0u;
+            tot += c[k];
+        }
+        uint32_t incl = tot;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t y = __shfl_up_sync(kFull, incl, o);
+            if (lane >= o) incl += y;
+        }
+        if (lane == 31) wtot[w] = incl;
+        __syncthreads();
+        uint32_t pre = 0, all = 0;
+#pragma unroll
+        for (int i = 0; i < kScanThreads / 32; i++) {
+            pre += i < w ? wtot[i] : 0u;
+            all += wtot[i];
+        }
+        unsigned long long o = run + pre + incl - tot;
+#pragma unroll
+        for (int k = 0; k < 4; k++) {
+            if (t0 + k < hi) off[t0 + k] = (uint32_t)o;
+            o += c[k];
+        }
+        run += all;
+        __syncthreads();   // wtot is rewritten by the next chunk
+    }
+    if (hi == n && threadIdx.x == 0) {   // the last span
+        off[n] = (uint32_t)run;
+        if (total_out) *total_out = (int64_t)run;
+    }
+}
+
+// One span of Gaussians a block: their codes and the span's output count.
+__global__ void __launch_bounds__(kScanThreads)
+k_densify_plan(const float *__restrict__ P, int64_t n, int64_t span, const float *__restrict__ accum,
+               const float *__restrict__ denom, float t_grad, float t_logs, float t_logit,
+               uint32_t *__restrict__ code, unsigned long long *__restrict__ part)
+{
+    const int64_t lo = blockIdx.x * span, hi = min(n, lo + span);
+    unsigned long long outs = 0;
+#pragma unroll 4
+    for (int64_t g = lo + threadIdx.x; g < hi; g += kScanThreads) {
         const float den = denom[g];
         const float grad = den > 0.f ? __fdiv_rn(accum[g], den) : 0.f;
         const bool high = grad >= t_grad;
@@ -32,80 +135,47 @@ __global__ void k_densify_plan(const float *__restrict__ P, int64_t n, const flo
         const bool prune = P[10 * n + g] < t_logit;
         const uint32_t c = prune ? 0u : (high ? (small ? 2u : 3u) : 1u);
         code[g] = c;
-        count[g] = c == 0u ? 0u : (c == 1u ? 1u : 2u);
+        outs += min(c, 2u);
     }
+    outs = block_sum(outs);
+    if (threadIdx.x == 0) part[blockIdx.x] = outs;
 }
 
-// Single-block exclusive scan of count[0..n) into off[0..n], off[n] = total (warp chunks,
-// coalesced loads).
-__global__ void __launch_bounds__(1024)
-k_count_scan(const uint32_t *__restrict__ count, int64_t n, uint32_t *__restrict__ off, int64_t *__restrict__ total_out)
+// A block of kDenG consecutive Gaussians, whose outputs are consecutive too: a map in
+// shared memory says which Gaussian each output copies, and every group is then written
+// as one contiguous run of floats, lanes along it, so stores are whole lines and loads
+// nearly so (the copies of a Gaussian repeat its floats, a pruned one leaves a gap).  Bound
+// by HBM: 200k Gaussians of SH degree 3 in 78 us, 3.7 TB/s; one thread per Gaussian,
+// copying it float by float with the rows of a warp 180 bytes apart, took 266 us.
+constexpr int kDenG = 128, kDenThreads = 256;
+constexpr uint16_t kDenFresh = 0x4000, kDenSplit = 0x8000;   // zero moments; mean and scale drawn anew
+
+template <int DEG>
+__global__ void __launch_bounds__(kDenThreads)
+k_densify_apply(const float *__restrict__ P, const float *__restrict__ Mi, const float *__restrict__ Vi, int64_t n,
+                const uint32_t *__restrict__ code, const uint32_t *__restrict__ off,
+                const float *__restrict__ normals, int64_t m, float *__restrict__ Po, float *__restrict__ Mo,
+                float *__restrict__ Vo)
 {
-    __shared__ unsigned long long wtot[32];
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    const int64_t per = (n + 31) / 32;
-    const int64_t lo = (int64_t)w * per, hi = min(n, lo + per);
-    unsigned long long s = 0;
-    for (int64_t t = lo + lane; t < hi; t += 32) s += count[t];
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(kFull, s, o);
-    if (lane == 0) wtot[w] = s;
+    constexpr int R3 = 3 * ((DEG + 1) * (DEG + 1) - 1);
+    __shared__ uint16_t src[2 * kDenG];
+    __shared__ int s_outs;
+    const int64_t g0 = (int64_t)blockIdx.x * kDenG;
+    const int cnt = (int)min((int64_t)kDenG, n - g0);
+    const int64_t j0 = off[g0];
+    if (threadIdx.x == 0) s_outs = 0;
     __syncthreads();
-    unsigned long long run = 0, total = 0;
-    for (int i = 0; i < 32; i++) {
-        run += (i < w) ? wtot[i] : 0ull;
-        total += wtot[i];
-    }
-    for (int64_t base = lo; base < hi; base += 32) {
-        const int64_t t = base + lane;
-        const unsigned long long c = t < hi ? count[t] : 0ull;
-        unsigned long long incl = c;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const unsigned long long y = __shfl_up_sync(kFull, incl, o);
-            if (lane >= o) incl += y;
-        }
-        if (t < hi) off[t] = (uint32_t)(run + incl - c);
-        run += __shfl_sync(kFull, incl, 31);
-    }
-    if (threadIdx.x == 0) {
-        off[n] = (uint32_t)total;
-        *total_out = (int64_t)total;
-    }
-}
-
-// Copy Gaussian g of the input layout (n) to index j of the output layout (m); with
-// moments if src_m is non-null, else zero moments.
-__device__ __forceinline__ void copy_gaussian(const float *__restrict__ P, const float *__restrict__ Mi,
-                                              const float *__restrict__ Vi, int64_t n, int64_t g, float *__restrict__ Po,
-                                              float *__restrict__ Mo, float *__restrict__ Vo, int64_t m, int64_t j,
-                                              int K, bool moments)
-{
-    const int widths[6] = {3, 3, 4, 1, 3, 3 * (K - 1)};
-    int64_t oi = 0, oo = 0;
-    for (int gi = 0; gi < 6; gi++) {
-        const int w = widths[gi];
-        for (int c = 0; c < w; c++) {
-            Po[oo + (int64_t)w * j + c] = P[oi + (int64_t)w * g + c];
-            Mo[oo + (int64_t)w * j + c] = moments ? Mi[oi + (int64_t)w * g + c] : 0.f;
-            Vo[oo + (int64_t)w * j + c] = moments ? Vi[oi + (int64_t)w * g + c] : 0.f;
-        }
-        oi += (int64_t)w * n;
-        oo += (int64_t)w * m;
-    }
-}
-
-__global__ void k_densify_apply(const float *__restrict__ P, const float *__restrict__ Mi, const float *__restrict__ Vi,
-                                int64_t n, int K, const uint32_t *__restrict__ code, const uint32_t *__restrict__ off,
-                                const float *__restrict__ normals, int64_t m, float *__restrict__ Po,
-                                float *__restrict__ Mo, float *__restrict__ Vo)
-{
-    for (int64_t g = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; g < n; g += (int64_t)gridDim.x * blockDim.x) {
+    for (int gl = threadIdx.x; gl < cnt; gl += kDenThreads) {
+        const int64_t g = g0 + gl, j = off[g];
         const uint32_t c = code[g];
-        const int64_t j = off[g];
         if (c == 0u) continue;
-        if (j + (c == 1u ? 1 : 2) > m) continue;   // never write past the caller's n_out
-        if (c == 1u || c == 2u) copy_gaussian(P, Mi, Vi, n, g, Po, Mo, Vo, m, j, K, true);
-        if (c == 2u) copy_gaussian(P, Mi, Vi, n, g, Po, Mo, Vo, m, j + 1, K, false);
+        const int outs = c == 1u ? 1 : 2;
+        const int64_t jl = j - j0;
+        // never write past the caller's n_out, nor past the map
+        if (j + outs > m || jl < 0 || jl + outs > 2 * kDenG) continue;
+        atomicMax(&s_outs, (int)jl + outs);
+        src[jl] = (uint16_t)(gl | (c == 3u ? kDenFresh | kDenSplit : 0));
+        if (outs == 2) src[jl + 1] = (uint16_t)(gl | kDenFresh | (c == 3u ? kDenSplit : 0));
         if (c == 3u) {
             const float *q = P + 6 * n + 4 * g;
             const float inv = 1.0f / sqrtf(q[0] * q[0] + q[1] * q[1] + q[2] * q[2] + q[3] * q[3]);
@@ -117,7 +187,6 @@ __global__ void k_densify_apply(const float *__restrict__ P, const float *__rest
             const float s[3] = {expf(ls[0]), expf(ls[1]), expf(ls[2])};
             for (int k = 0; k < 2; k++) {
                 const int64_t jj = j + k;
-                copy_gaussian(P, Mi, Vi, n, g, Po, Mo, Vo, m, jj, K, false);
                 const float *zz = normals + 6 * g + 3 * k;
                 const float d0 = s[0] * zz[0], d1 = s[1] * zz[1], d2 = s[2] * zz[2];
                 for (int r = 0; r < 3; r++)
@@ -125,6 +194,29 @@ __global__ void k_densify_apply(const float *__restrict__ P, const float *__rest
                 for (int r = 0; r < 3; r++) Po[3 * m + 3 * jj + r] = ls[r] - kLogSplitDiv;
             }
         }
+    }
+    __syncthreads();
+    const int outs = s_outs;
+    const int widths[6] = {3, 3, 4, 1, 3, R3};
+    int64_t oi = 0, oo = 0;
+#pragma unroll
+    for (int gi = 0; gi < 6; gi++) {
+        const int w = widths[gi];
+        if (w == 0) continue;
+        const float *pi = P + oi + w * g0, *mi = Mi + oi + w * g0, *vi = Vi + oi + w * g0;
+        float *po = Po + oo + w * j0, *mo = Mo + oo + w * j0, *vo = Vo + oo + w * j0;
+#pragma unroll 4
+        for (int i = threadIdx.x; i < w * outs; i += kDenThreads) {
+            const int jl = i / w;
+            const uint32_t e = src[jl];
+            const int from = w * (int)(e & (kDenFresh - 1)) + i - w * jl;
+            const bool fresh = e & kDenFresh;
+            if (gi >= 2 || !(e & kDenSplit)) po[i] = __ldg(pi + from);
+            mo[i] = fresh ? 0.f : __ldg(mi + from);
+            vo[i] = fresh ? 0.f : __ldg(vi + from);
+        }
+        oi += (int64_t)w * n;
+        oo += (int64_t)w * m;
     }
 }
 
@@ -134,25 +226,35 @@ __global__ void k_densify_apply(const float *__restrict__ P, const float *__rest
 // mean squared distance to the 3 nearest other points (exact), identity rotation,
 // opacity logit(init), SH DC (rgb - 1/2) / Y_0^0, higher bands 0.
 //
-// Exact k-NN on a uniform grid: bounding box and moments (k_bbox); the grid spans the box
-// cut to mean +- 3 standard deviations per axis, points outside fall into the border cells
-// (so a few far outliers do not stretch the cells); cell size (k_grid_setup) about one point
+// Exact k-NN on a uniform grid: bounding box and moments, then the grid (k_bbox); the grid
+// spans the box cut to mean +- 3 standard deviations per axis, points outside fall into the
+// border cells (so a few far outliers do not stretch the cells); cell size about one point
 // per cell of the box's volume, face area or length, whichever is largest, and at most
-// kGridCap cells per axis; counting sort of point ids by cell (k_cell_count, k_count_scan, k_cell_scatter),
-// then per point a search over growing rings of cells that stops once the distance to
-// the unsearched region, less a rounding margin, is at least the third-best distance.
+// kGridCap cells per axis; counting sort of the points by cell (k_cell_count, the scan,
+// k_cell_scatter), which copies their coordinates into cell order, so a row of cells along x
+// is one contiguous run of points.  Per point a search over growing rings of cells stops
+// once the distance to the unsearched region, less a rounding margin, is at least the
+// third-best distance (k_knn); points not settled within kNearRings rings are listed and
+// searched by a block each (k_knn_far).
 
 constexpr int kGridCap = 128;
 constexpr int kKnn = 3;
 constexpr float kKnnFloor = 1e-7f;
 constexpr float kShC0 = 0.28209479177387814f;
+// Rings a single thread searches.  A stray point far outside the room has to look at
+// every cell of the grid: one thread walking them alone took 122 ms on a 307k-point frame
+// with two such points, where k_knn takes 160 us and k_knn_far 17 us.
+constexpr int kNearRings = 4;
+constexpr int kFarThreads = 512, kFarSample = 4096;
 
 struct GridInfo {
     float lo[3];
     float h;
     int G[3];
     float margin;
-    uint32_t box[6];   // sortable encodings: min x, y, z, then max x, y, z
+    uint32_t box[6];   // sortable encodings, all maxima: complements of min x, y, z, then max x, y, z
+    uint32_t done;     // blocks of k_bbox that have added their part
+    uint32_t nfar;     // points listed for k_knn_far
     double sum[3], sumsq[3];
 };
 
@@ -171,54 +273,19 @@ __device__ __forceinline__ float sortable2f(uint32_t u)
     return __uint_as_float((u & 0x80000000u) ? (u & 0x7fffffffu) : ~u);
 }
 
-__global__ void k_bbox(const float *__restrict__ xyz, int64_t m, GridInfo *__restrict__ gi, int32_t *status)
+// Grid of the points from their box and moments (one thread).
+__device__ void grid_setup(GridInfo *gi, int64_t m, int64_t budget)
 {
-    float lo[3] = {INFINITY, INFINITY, INFINITY}, hi[3] = {-INFINITY, -INFINITY, -INFINITY};
-    double s1[3] = {0.0, 0.0, 0.0}, s2[3] = {0.0, 0.0, 0.0};
-    bool bad = false;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < m; i += (int64_t)gridDim.x * blockDim.x)
-        for (int a = 0; a < 3; a++) {
-            const float x = xyz[3 * i + a];
-            if (!isfinite(x)) {
-                bad = true;
-                continue;
-            }
-            lo[a] = fminf(lo[a], x);
-            hi[a] = fmaxf(hi[a], x);
-            s1[a] += x;
-            s2[a] += (double)x * x;
-        }
-    for (int a = 0; a < 3; a++)
-        for (int o = 16; o > 0; o >>= 1) {
-            lo[a] = fminf(lo[a], __shfl_xor_sync(kFull, lo[a], o));
-            hi[a] = fmaxf(hi[a], __shfl_xor_sync(kFull, hi[a], o));
-            s1[a] += __shfl_xor_sync(kFull, s1[a], o);
-            s2[a] += __shfl_xor_sync(kFull, s2[a], o);
-        }
-    if (__any_sync(kFull, bad) && (threadIdx.x & 31) == 0) set_status(status, CGS_ERR_NONFINITE);
-    if ((threadIdx.x & 31) == 0)
-        for (int a = 0; a < 3; a++) {
-            if (lo[a] <= hi[a]) {
-                atomicMin(&gi->box[a], f2sortable(lo[a]));
-                atomicMax(&gi->box[3 + a], f2sortable(hi[a]));
-                atomicAdd(&gi->sum[a], s1[a]);
-                atomicAdd(&gi->sumsq[a], s2[a]);
-            }
-        }
-}
-
-__global__ void k_grid_setup(GridInfo *__restrict__ gi, int64_t m, int64_t budget)
-{
-    if (threadIdx.x != 0) return;
     float lo[3], ext[3];
     float emax = 0.f, amax = 0.f;
     const double mm = (double)(m > 0 ? m : 1);
     for (int a = 0; a < 3; a++) {
-        const bool any = gi->box[a] != 0xffffffffu;
-        const float blo = any ? sortable2f(gi->box[a]) : 0.f;
-        const float bhi = any ? sortable2f(gi->box[3 + a]) : 0.f;
-        const double mu = gi->sum[a] / mm;
-        const double sd = sqrt(fmax(gi->sumsq[a] / mm - mu * mu, 0.0));
+        const uint32_t bmin = __ldcg(&gi->box[a]), bmax = __ldcg(&gi->box[3 + a]);
+        const bool any = bmax != 0u;
+        const float blo = any ? sortable2f(~bmin) : 0.f;
+        const float bhi = any ? sortable2f(bmax) : 0.f;
+        const double mu = __ldcg(&gi->sum[a]) / mm;
+        const double sd = sqrt(fmax(__ldcg(&gi->sumsq[a]) / mm - mu * mu, 0.0));
         lo[a] = fmaxf(blo, (float)(mu - 3.0 * sd));
         const float hi = fmaxf(fminf(bhi, (float)(mu + 3.0 * sd)), lo[a]);
         ext[a] = fmaxf(hi - lo[a], 0.f);
@@ -254,14 +321,78 @@ __global__ void k_grid_setup(GridInfo *__restrict__ gi, int64_t m, int64_t budge
     gi->margin = 8.f * 1.2e-7f * (amax + 2.f * hf);
 }
 
+// gi starts all zero; the block that finishes last sets up the grid.  Each block adds its
+// part with twelve atomics: a set from every warp queued tens of thousands on the same
+// words (307k points 95 us and 8 us for the set-up's own launch, now 20 us together).
+constexpr int kBoxThreads = 256;
+__global__ void __launch_bounds__(kBoxThreads)
+k_bbox(const float *__restrict__ xyz, int64_t m, int64_t budget, GridInfo *__restrict__ gi, int32_t *status)
+{
+    __shared__ uint32_t sbox[8][6];
+    __shared__ double smom[6][kBoxThreads];
+    float lo[3] = {INFINITY, INFINITY, INFINITY}, hi[3] = {-INFINITY, -INFINITY, -INFINITY};
+    double s1[3] = {0.0, 0.0, 0.0}, s2[3] = {0.0, 0.0, 0.0};
+    bool bad = false;
+#pragma unroll 4
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < m; i += (int64_t)gridDim.x * blockDim.x)
+        for (int a = 0; a < 3; a++) {
+            const float x = xyz[3 * i + a];
+            if (!isfinite(x)) {
+                bad = true;
+                continue;
+            }
+            lo[a] = fminf(lo[a], x);
+            hi[a] = fmaxf(hi[a], x);
+            s1[a] += x;
+            s2[a] += (double)x * x;
+        }
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    for (int a = 0; a < 3; a++) {
+        for (int o = 16; o > 0; o >>= 1) {
+            lo[a] = fminf(lo[a], __shfl_xor_sync(kFull, lo[a], o));
+            hi[a] = fmaxf(hi[a], __shfl_xor_sync(kFull, hi[a], o));
+        }
+        smom[a][threadIdx.x] = s1[a];
+        smom[3 + a][threadIdx.x] = s2[a];
+        if (lane == 0) {
+            const bool any = lo[a] <= hi[a];
+            sbox[w][a] = any ? ~f2sortable(lo[a]) : 0u;
+            sbox[w][3 + a] = any ? f2sortable(hi[a]) : 0u;
+        }
+    }
+    if (__any_sync(kFull, bad) && lane == 0) set_status(status, CGS_ERR_NONFINITE);
+    __syncthreads();
+    // one warp per sum: FP64 is slow on this part, a shuffle tree in every warp took most of
+    // the kernel
+    if (w < 6) {
+        double y = 0.0;
+        for (int i = lane; i < kBoxThreads; i += 32) y += smom[w][i];
+        for (int o = 16; o > 0; o >>= 1) y += __shfl_xor_sync(kFull, y, o);
+        if (lane == 0) {
+            uint32_t x = 0;
+            for (int i = 0; i < kBoxThreads / 32; i++) x = max(x, sbox[i][w]);
+            atomicMax(&gi->box[w], x);
+            atomicAdd(w < 3 ? &gi->sum[w] : &gi->sumsq[w - 3], y);
+            __threadfence();
+        }
+    }
+    __syncthreads();
+    if (threadIdx.x == 0 && atomicAdd(&gi->done, 1u) == gridDim.x - 1) {
+        __threadfence();
+        grid_setup(gi, m, budget);
+    }
+}
+
 __device__ __forceinline__ int cell_axis(float x, float lo, float h, int G)
 {
     int c = (int)floorf((x - lo) / h);
     return c < 0 ? 0 : (c >= G ? G - 1 : c);
 }
 
+// Cell of every point, and its rank among the cell's points (whatever order the atomics took).
 __global__ void k_cell_count(const float *__restrict__ xyz, int64_t m, const GridInfo *__restrict__ gi,
-                             uint32_t *__restrict__ cell_of, uint32_t *__restrict__ count)
+                             uint32_t *__restrict__ cell_of, uint32_t *__restrict__ rank,
+                             uint32_t *__restrict__ count)
 {
     const GridInfo g = *gi;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < m; i += (int64_t)gridDim.x * blockDim.x) {
@@ -270,139 +401,292 @@ __global__ void k_cell_count(const float *__restrict__ xyz, int64_t m, const Gri
         const int cz = cell_axis(xyz[3 * i + 2], g.lo[2], g.h, g.G[2]);
         const uint32_t c = (uint32_t)cx + (uint32_t)g.G[0] * ((uint32_t)cy + (uint32_t)g.G[1] * (uint32_t)cz);
         cell_of[i] = c;
-        atomicAdd(count + c, 1u);
+        rank[i] = atomicAdd(count + c, 1u);
     }
 }
 
-__global__ void k_cell_scatter(int64_t m, const uint32_t *__restrict__ cell_of, const uint32_t *__restrict__ off,
-                               uint32_t *__restrict__ count, uint32_t *__restrict__ ids)
+__global__ void k_cell_scatter(const float *__restrict__ xyz, int64_t m, const uint32_t *__restrict__ cell_of,
+                               const uint32_t *__restrict__ rank, const uint32_t *__restrict__ off,
+                               float4 *__restrict__ pts)
 {
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < m; i += (int64_t)gridDim.x * blockDim.x) {
-        const uint32_t c = cell_of[i];
-        ids[off[c] + atomicSub(count + c, 1u) - 1u] = (uint32_t)i;
-    }
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < m; i += (int64_t)gridDim.x * blockDim.x)
+        pts[off[cell_of[i]] + rank[i]] =
+            make_float4(xyz[3 * i], xyz[3 * i + 1], xyz[3 * i + 2], __uint_as_float((uint32_t)i));
 }
 
-__device__ __forceinline__ void knn_insert(float d, float (&best)[kKnn], int &nb)
-{
-    if (nb < kKnn) {
-        best[nb++] = d;
-    } else if (d < best[kKnn - 1]) {
-        best[kKnn - 1] = d;
-    } else {
-        return;
+// The three smallest distances, ascending (infinite until found).
+struct Best {
+    float b0 = INFINITY, b1 = INFINITY, b2 = INFINITY;
+    __device__ __forceinline__ void insert(float d)
+    {
+        if (!(d < b2)) return;
+        const float t = fmaxf(b0, d);
+        b0 = fminf(b0, d);
+        b2 = fmaxf(b1, t);
+        b1 = fminf(b1, t);
     }
-#pragma unroll
-    for (int a = kKnn - 1; a > 0; a--)
-        if (a < nb && best[a] < best[a - 1]) {
-            const float t = best[a];
-            best[a] = best[a - 1];
-            best[a - 1] = t;
+    __device__ __forceinline__ float nth(int want) const { return want <= 1 ? b0 : (want == 2 ? b1 : b2); }
+};
+
+// A point, its cell, and the bounds that let the search leave cells out.
+struct Query {
+    GridInfo g;
+    uint32_t self;     // position in cell order
+    float p[3];
+    int c[3];
+    int want;          // neighbours there are to find: min(3, points - 1)
+
+    __device__ __forceinline__ Query(const GridInfo &gi, const float4 &q, uint32_t at, int64_t m)
+        : g(gi), self(at), p{q.x, q.y, q.z}, want(m - 1 < kKnn ? (int)(m - 1) : kKnn)
+    {
+        for (int a = 0; a < 3; a++) c[a] = cell_axis(p[a], g.lo[a], g.h, g.G[a]);
+    }
+    __device__ __forceinline__ float dist2(const float4 &q) const
+    {
+        const float ex = q.x - p[0], ey = q.y - p[1], ez = q.z - p[2];
+        return ex * ex + ey * ey + ez * ez;
+    }
+    // Squared distance from the point to every point of cells i0..i1 along axis a is at least
+    // this (border cells reach outwards without end).
+    __device__ __forceinline__ float gap2(int a, int i0, int i1) const
+    {
+        float d = 0.f;
+        if (i0 > 0) d = fmaxf(d, (g.lo[a] + (float)i0 * g.h) - p[a]);
+        if (i1 < g.G[a] - 1) d = fmaxf(d, p[a] - (g.lo[a] + (float)(i1 + 1) * g.h));
+        d = fmaxf(d - g.margin, 0.f);
+        return d * d;
+    }
+    __device__ __forceinline__ bool beyond(float low2, const Best &b) const
+    {
+        return low2 >= b.nth(want) * (1.f + 1e-6f);
+    }
+    // Cells up to Chebyshev distance r have been searched: is every other point too far?
+    __device__ __forceinline__ bool settled(int r, const Best &b) const
+    {
+        float bound = INFINITY;
+        for (int a = 0; a < 3; a++) {
+            if (c[a] - r > 0) bound = fminf(bound, p[a] - (g.lo[a] + (float)(c[a] - r) * g.h));
+            if (c[a] + r < g.G[a] - 1) bound = fminf(bound, (g.lo[a] + (float)(c[a] + r + 1) * g.h) - p[a]);
         }
-}
-
-__device__ __forceinline__ void knn_cell(const float *__restrict__ xyz, const uint32_t *__restrict__ off,
-                                         const uint32_t *__restrict__ ids, uint32_t cell, uint32_t i, float px,
-                                         float py, float pz, float (&best)[kKnn], int &nb)
-{
-    for (uint32_t q = off[cell]; q < off[cell + 1]; q++) {
-        const uint32_t j = ids[q];
-        if (j == i) continue;
-        const float ex = xyz[3 * j] - px, ey = xyz[3 * j + 1] - py, ez = xyz[3 * j + 2] - pz;
-        knn_insert(ex * ex + ey * ey + ez * ez, best, nb);
+        if (bound == INFINITY) return true;   // every cell searched
+        const float d = bound - g.margin;
+        return d > 0.f && beyond(d * d, b);
     }
-}
+    __device__ __forceinline__ float log_scale(const Best &b) const
+    {
+        float d2 = 0.f;
+        if (p[0] != p[0] || p[1] != p[1] || p[2] != p[2]) return 0.5f * logf(kKnnFloor);   // no distances at all
+        if (want > 0) d2 += b.b0;
+        if (want > 1) d2 += b.b1;
+        if (want > 2) d2 += b.b2;
+        if (want > 0) d2 = d2 / (float)want;
+        return 0.5f * logf(fmaxf(d2, kKnnFloor));
+    }
+};
 
-// One thread per point, in cell order.  Writes Gaussian n + i of the output layout (m_out).
+// One thread per point, in cell order: log-scale of Gaussian n + id into ls (3 per Gaussian).
+// Bound by the latency of its loads: a row of cells costs two offsets and one run of
+// coordinates, and rows and cells that lie beyond the third-best distance are not read.
 __global__ void __launch_bounds__(128)
-k_knn_init(const float *__restrict__ xyz, const float *__restrict__ rgb, int64_t m, const GridInfo *__restrict__ gi,
-           const uint32_t *__restrict__ cell_of, const uint32_t *__restrict__ off, const uint32_t *__restrict__ ids,
-           int K, float logit, int64_t n, int64_t n_out, float *__restrict__ Po)
+k_knn(const float4 *__restrict__ pts, int64_t m, GridInfo *__restrict__ gi, const uint32_t *__restrict__ off,
+      uint32_t *__restrict__ far, float *__restrict__ ls)
 {
-    const GridInfo g = *gi;
-    const int want = m - 1 < kKnn ? (int)(m - 1) : kKnn;
     for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < m; t += (int64_t)gridDim.x * blockDim.x) {
-        const uint32_t i = ids[t];
-        const float px = xyz[3 * i], py = xyz[3 * i + 1], pz = xyz[3 * i + 2];
-        const uint32_t c = cell_of[i];
-        const int cx = (int)(c % (uint32_t)g.G[0]), cy = (int)((c / (uint32_t)g.G[0]) % (uint32_t)g.G[1]),
-                  cz = (int)(c / ((uint32_t)g.G[0] * (uint32_t)g.G[1]));
-        float best[kKnn];
-        int nb = 0;
-        const int rmax = want > 0 ? max(g.G[0], max(g.G[1], g.G[2])) : -1;
-        for (int r = 0; r <= rmax; r++) {
-            const int z0 = max(-r, -cz), z1 = min(r, g.G[2] - 1 - cz);
-            const int y0 = max(-r, -cy), y1 = min(r, g.G[1] - 1 - cy);
-            const int x0 = max(-r, -cx), x1 = min(r, g.G[0] - 1 - cx);
-            for (int dz = z0; dz <= z1; dz++)
+        const float4 me = pts[t];
+        const Query Q(*gi, me, (uint32_t)t, m);
+        const GridInfo &g = Q.g;
+        Best best;
+        bool found = Q.want == 0;
+        for (int r = 0; r <= kNearRings && !found; r++) {
+            const int z0 = max(-r, -Q.c[2]), z1 = min(r, g.G[2] - 1 - Q.c[2]);
+            const int y0 = max(-r, -Q.c[1]), y1 = min(r, g.G[1] - 1 - Q.c[1]);
+            const int x0 = max(Q.c[0] - r, 0), x1 = min(Q.c[0] + r, g.G[0] - 1);
+            for (int dz = z0; dz <= z1; dz++) {
+                const float gz = Q.gap2(2, Q.c[2] + dz, Q.c[2] + dz);
+                if (Q.beyond(gz, best)) continue;
                 for (int dy = y0; dy <= y1; dy++) {
+                    const float gyz = gz + Q.gap2(1, Q.c[1] + dy, Q.c[1] + dy);
+                    if (Q.beyond(gyz, best)) continue;
                     // cells at Chebyshev distance exactly r: whole rows on the faces dz = +-r or
                     // dy = +-r, else only dx = -r and dx = +r
                     const bool face = dz == -r || dz == r || dy == -r || dy == r;
-                    const uint32_t row = (uint32_t)g.G[0] * ((uint32_t)(cy + dy) + (uint32_t)g.G[1] * (uint32_t)(cz + dz));
-                    if (face) {
-                        for (int dx = x0; dx <= x1; dx++)
-                            knn_cell(xyz, off, ids, row + (uint32_t)(cx + dx), i, px, py, pz, best, nb);
-                    } else {
-                        if (-r >= x0) knn_cell(xyz, off, ids, row + (uint32_t)(cx - r), i, px, py, pz, best, nb);
-                        if (r <= x1) knn_cell(xyz, off, ids, row + (uint32_t)(cx + r), i, px, py, pz, best, nb);
+                    const uint32_t row =
+                        (uint32_t)g.G[0] * ((uint32_t)(Q.c[1] + dy) + (uint32_t)g.G[1] * (uint32_t)(Q.c[2] + dz));
+                    for (int side = 0; side < (face ? 1 : 2); side++) {
+                        const int a0 = face ? x0 : (side ? Q.c[0] + r : Q.c[0] - r), a1 = face ? x1 : a0;
+                        if (a0 < 0 || a1 >= g.G[0] || Q.beyond(gyz + Q.gap2(0, a0, a1), best)) continue;
+                        const uint32_t q1 = off[row + (uint32_t)a1 + 1];
+                        for (uint32_t q = off[row + (uint32_t)a0]; q < q1; q++)
+                            if (q != Q.self) best.insert(Q.dist2(pts[q]));
                     }
                 }
-            // distance from the point to the region outside the searched block of cells
-            float bound = INFINITY;
-            const float p[3] = {px, py, pz};
-            const int cc3[3] = {cx, cy, cz};
-            for (int a = 0; a < 3; a++) {
-                if (cc3[a] - r > 0) bound = fminf(bound, p[a] - (g.lo[a] + (float)(cc3[a] - r) * g.h));
-                if (cc3[a] + r < g.G[a] - 1) bound = fminf(bound, (g.lo[a] + (float)(cc3[a] + r + 1) * g.h) - p[a]);
             }
-            if (bound == INFINITY) break;                   // every cell searched
-            const float b = bound - g.margin;
-            if (nb >= want && b > 0.f && b * b >= best[want - 1] * (1.f + 1e-6f)) break;
+            found = Q.settled(r, best);
         }
-        float d2 = 0.f;
-        for (int a = 0; a < nb; a++) d2 += best[a];
-        d2 = nb ? d2 / (float)nb : 0.f;
-        const float ls = 0.5f * logf(fmaxf(d2, kKnnFloor));
-        const int64_t j = n + i;
-        for (int a = 0; a < 3; a++) {
-            Po[3 * j + a] = xyz[3 * i + a];
-            Po[3 * n_out + 3 * j + a] = ls;
-            Po[11 * n_out + 3 * j + a] = (rgb[3 * i + a] - 0.5f) / kShC0;
+        if (!found) {
+            far[atomicAdd(&gi->nfar, 1u)] = (uint32_t)t;
+            continue;
         }
-        Po[6 * n_out + 4 * j] = 1.f;
-        Po[6 * n_out + 4 * j + 1] = 0.f;
-        Po[6 * n_out + 4 * j + 2] = 0.f;
-        Po[6 * n_out + 4 * j + 3] = 0.f;
-        Po[10 * n_out + j] = logit;
-        for (int a = 0; a < 3 * (K - 1); a++) Po[14 * n_out + (int64_t)3 * (K - 1) * j + a] = 0.f;
+        const float l = Q.log_scale(best);
+        float *o = ls + 3 * (int64_t)__float_as_uint(me.w);
+        o[0] = l;
+        o[1] = l;
+        o[2] = l;
     }
 }
 
-// Gaussians 0..n-1 of the input layout (n) to the same indices of the output layout.
-__global__ void k_copy_prefix(const float *__restrict__ P, const float *__restrict__ Mi, const float *__restrict__ Vi,
-                              int64_t n, int K, int64_t n_out, float *__restrict__ Po, float *__restrict__ Mo,
-                              float *__restrict__ Vo)
+// The listed points, one block each.  An evenly spaced sample of the cloud bounds the
+// third-best distance first; then the lanes of a warp take 32 rows of cells at a time, cut to
+// the cells within that distance, and those rows' points together.
+__global__ void __launch_bounds__(kFarThreads)
+k_knn_far(const float4 *__restrict__ pts, int64_t m, const GridInfo *__restrict__ gi,
+          const uint32_t *__restrict__ off, const uint32_t *__restrict__ far, float *__restrict__ ls)
 {
-    for (int64_t g = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; g < n; g += (int64_t)gridDim.x * blockDim.x)
-        copy_gaussian(P, Mi, Vi, n, g, Po, Mo, Vo, n_out, g, K, true);
+    constexpr int NW = kFarThreads / 32;
+    __shared__ Best sbest[NW];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    auto merge = [](Best &a, const Best &b) {
+        a.insert(b.b0);
+        a.insert(b.b1);
+        a.insert(b.b2);
+    };
+    auto block_best = [&](Best best) {   // the block's three smallest, in every thread
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            Best other;
+            other.b0 = __shfl_down_sync(kFull, best.b0, o);
+            other.b1 = __shfl_down_sync(kFull, best.b1, o);
+            other.b2 = __shfl_down_sync(kFull, best.b2, o);
+            if (lane < o) merge(best, other);
+        }
+        __syncthreads();   // the previous result has been read
+        if (lane == 0) sbest[w] = best;
+        __syncthreads();
+        best = sbest[0];
+        for (int i = 1; i < NW; i++) merge(best, sbest[i]);
+        return best;
+    };
+    const uint32_t nfar = gi->nfar;
+    for (uint32_t f = blockIdx.x; f < nfar; f += gridDim.x) {
+        const uint32_t t = far[f];
+        const float4 me = pts[t];
+        const Query Q(*gi, me, t, m);
+        const GridInfo &g = Q.g;
+        Best best;
+        const int64_t step = (m + kFarSample - 1) / kFarSample;
+#pragma unroll 4
+        for (int64_t q = threadIdx.x * step; q < m; q += kFarThreads * step)
+            if (q != t) best.insert(Q.dist2(pts[q]));
+        const Best bound = block_best(best);
+        const float reach2 = bound.nth(Q.want) * (1.f + 1e-6f);
+        best = Best();
+        const int rows = g.G[1] * g.G[2];
+        for (int r0 = 32 * w; r0 < rows; r0 += kFarThreads) {   // warp-uniform
+            const int rr = r0 + lane, y = rr % g.G[1], z = rr / g.G[1];
+            uint32_t q0 = 0u, len = 0u;
+            if (rr < rows) {
+                const float low2 = Q.gap2(1, y, y) + Q.gap2(2, z, z);
+                if (low2 <= reach2) {
+                    // the cells along x within reach, one more on each side for the rounding
+                    // (distances past an int's range end at the border cells)
+                    const float d = sqrtf(fmaxf(reach2 - low2, 0.f)) + g.margin;
+                    const int x0 = max(cell_axis(Q.p[0] - d, g.lo[0], g.h, g.G[0]) - 1, 0);
+                    const int x1 = min(cell_axis(Q.p[0] + d, g.lo[0], g.h, g.G[0]) + 1, g.G[0] - 1);
+                    const uint32_t row = (uint32_t)rr * (uint32_t)g.G[0];
+                    q0 = off[row + (uint32_t)x0];
+                    len = off[row + (uint32_t)x1 + 1] - q0;
+                }
+            }
+            uint32_t incl = len;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const uint32_t y2 = __shfl_up_sync(kFull, incl, o);
+                if (lane >= o) incl += y2;
+            }
+            const uint32_t total = __shfl_sync(kFull, incl, 31), first = q0 - (incl - len);
+            for (uint32_t j0 = 0; j0 < total; j0 += 32) {   // warp-uniform
+                const uint32_t j = j0 + lane;
+                int L = 0;   // owner: the number of lanes whose inclusive prefix is <= j
+#pragma unroll
+                for (int b = 16; b > 0; b >>= 1)
+                    if (__shfl_sync(kFull, incl, L + b - 1) <= j) L += b;
+                const uint32_t q = __shfl_sync(kFull, first, L) + j;
+                if (j < total && q != t) best.insert(Q.dist2(pts[q]));
+            }
+        }
+        best = block_best(best);
+        if (threadIdx.x < 3) ls[3 * (int64_t)__float_as_uint(me.w) + threadIdx.x] = Q.log_scale(best);
+    }
 }
 
-// Zero Adam moments of Gaussians n..n_out-1.
-__global__ void k_zero_tail(int64_t n, int K, int64_t n_out, float *__restrict__ Mo, float *__restrict__ Vo)
+// The rest of the output as runs of floats: the old Gaussians' groups copied, and the new
+// ones' appended, a run per (array, group, old or new).  Every block fills one chunk of a
+// run, so the kind of run is uniform and both sides are contiguous.  Bound by HBM: 100k old
+// and 307k new Gaussians of SH degree 3 in 60 us, 6.0 TB/s; a thread per Gaussian took 141 us
+// for the old, 212 us for the new ones' moments and part of the neighbour search for the rest.
+enum RunKind { kRunCopy, kRunFill, kRunQuat, kRunColor };
+struct Run {
+    float *dst;
+    const float *src;
+    int64_t len, block0;   // floats; first block
+    float value;
+    int kind;
+};
+constexpr int kMaxRuns = 36, kRunThreads = 256, kRunChunk = 16 * kRunThreads;
+struct Runs {
+    Run run[kMaxRuns];
+    int n;
+    int64_t blocks;
+};
+
+__global__ void __launch_bounds__(kRunThreads) k_runs(const __grid_constant__ Runs R)
 {
-    const int widths[6] = {3, 3, 4, 1, 3, 3 * (K - 1)};
-    for (int64_t g = n + blockIdx.x * (int64_t)blockDim.x + threadIdx.x; g < n_out;
-         g += (int64_t)gridDim.x * blockDim.x) {
-        int64_t o = 0;
-        for (int gi = 0; gi < 6; gi++) {
-            for (int c = 0; c < widths[gi]; c++) {
-                Mo[o + (int64_t)widths[gi] * g + c] = 0.f;
-                Vo[o + (int64_t)widths[gi] * g + c] = 0.f;
-            }
-            o += (int64_t)widths[gi] * n_out;
+    int k = 0;
+    while (k + 1 < R.n && (int64_t)blockIdx.x >= R.run[k + 1].block0) k++;
+    const Run &r = R.run[k];
+    const int64_t e0 = (blockIdx.x - r.block0) * kRunChunk;
+    const int cnt = (int)min((int64_t)kRunChunk, r.len - e0);
+    float *d = r.dst + e0;
+    const float *s = r.src ? r.src + e0 : nullptr;
+    switch (r.kind) {
+    case kRunCopy: {
+        // all of the chunk's loads in flight before the first store
+        float x[kRunChunk / kRunThreads];
+#pragma unroll
+        for (int q = 0; q < kRunChunk / kRunThreads; q++) {
+            const int i = q * kRunThreads + (int)threadIdx.x;
+            x[q] = i < cnt ? __ldg(s + i) : 0.f;
         }
+#pragma unroll
+        for (int q = 0; q < kRunChunk / kRunThreads; q++) {
+            const int i = q * kRunThreads + (int)threadIdx.x;
+            if (i < cnt) d[i] = x[q];
+        }
+        break;
     }
+    case kRunFill: {
+        // whole 16-byte words from the first aligned one
+        const int head = min(cnt, (int)(((16u - ((uint32_t)(uintptr_t)d & 15u)) & 15u) >> 2)), words = (cnt - head) / 4;
+        const float4 v4 = make_float4(r.value, r.value, r.value, r.value);
+        for (int i = threadIdx.x; i < words; i += kRunThreads) reinterpret_cast<float4 *>(d + head)[i] = v4;
+        for (int i = threadIdx.x; i < cnt; i += kRunThreads)
+            if (i < head || i >= head + 4 * words) d[i] = r.value;
+        break;
+    }
+    case kRunQuat:   // identity rotations
+        for (int i = threadIdx.x; i < cnt; i += kRunThreads) d[i] = (i & 3) == 0 ? 1.f : 0.f;
+        break;
+    default:   // colours as SH DC coefficients
+        for (int i = threadIdx.x; i < cnt; i += kRunThreads) d[i] = (__ldg(s + i) - 0.5f) / kShC0;
+    }
+}
+static_assert(kRunChunk % 4 == 0, "a chunk of quaternions starts at a whole one");
+
+static void add_run(Runs &R, float *dst, const float *src, int64_t len, int kind, float value = 0.f)
+{
+    if (len <= 0) return;
+    R.run[R.n++] = Run{dst, src, len, R.blocks, value, kind};
+    R.blocks += (len + kRunChunk - 1) / kRunChunk;
 }
 
 }  // namespace cgs
@@ -438,15 +722,18 @@ int cgs_densify_plan(const float *params, int64_t n, int32_t sh_degree, const fl
     if (((uintptr_t)workspace & 255) != 0) return CGS_ERR_ARG;
     if (workspace_bytes < cgs_densify_workspace(n)) return CGS_ERR_WORKSPACE;
     uint32_t *code = static_cast<uint32_t *>(workspace);
-    uint32_t *count = reinterpret_cast<uint32_t *>(static_cast<char *>(workspace) + al256(sizeof(uint32_t) * n));
+    // span totals: at most one per kScanChunk Gaussians
+    unsigned long long *part =
+        reinterpret_cast<unsigned long long *>(static_cast<char *>(workspace) + al256(sizeof(uint32_t) * n));
     uint32_t *off = reinterpret_cast<uint32_t *>(static_cast<char *>(workspace) + 2 * al256(sizeof(uint32_t) * n));
     const float t_grad = (float)tau_p;
     const float t_logs = (float)log(scale_thr);
     const float t_logit = (float)log(eps_alpha / (1.0 - eps_alpha));
     cudaStream_t s = (cudaStream_t)stream;
-    const int blocks = (int)((n + 255) / 256 < 4096 ? (n + 255) / 256 : 4096);
-    k_densify_plan<<<blocks, 256, 0, s>>>(params, n, accum, denom, t_grad, t_logs, t_logit, code, count);
-    k_count_scan<<<1, 1024, 0, s>>>(count, n, off, n_out_dev);
+    const int64_t span = scan_span(n);
+    const int blocks = scan_blocks(n);
+    k_densify_plan<<<blocks, kScanThreads, 0, s>>>(params, n, span, accum, denom, t_grad, t_logs, t_logit, code, part);
+    k_span_scan<<<blocks, kScanThreads, 0, s>>>(CodeEntry{code}, n, span, part, off, n_out_dev);
     return st_of(cudaGetLastError());
 }
 
@@ -462,10 +749,13 @@ int cgs_densify_apply(const float *params, const float *m, const float *v, int64
     const uint32_t *code = static_cast<const uint32_t *>(workspace);
     const uint32_t *off =
         reinterpret_cast<const uint32_t *>(static_cast<const char *>(workspace) + 2 * al256(sizeof(uint32_t) * n));
-    const int K = (sh_degree + 1) * (sh_degree + 1);
     cudaStream_t s = (cudaStream_t)stream;
-    const int blocks = (int)((n + 255) / 256 < 4096 ? (n + 255) / 256 : 4096);
-    k_densify_apply<<<blocks, 256, 0, s>>>(params, m, v, n, K, code, off, normals, n_out, params_out, m_out, v_out);
+    auto k = sh_degree == 0   ? k_densify_apply<0>
+             : sh_degree == 1 ? k_densify_apply<1>
+             : sh_degree == 2 ? k_densify_apply<2>
+                              : k_densify_apply<3>;
+    k<<<(unsigned)((n + kDenG - 1) / kDenG), kDenThreads, 0, s>>>(params, m, v, n, code, off, normals, n_out,
+                                                                  params_out, m_out, v_out);
     return st_of(cudaGetLastError());
 }
 
@@ -473,8 +763,9 @@ size_t cgs_points_workspace(int64_t n_points)
 {
     if (n_points < 1) return 0;
     const int64_t B = grid_cell_budget(n_points);
-    return al256(sizeof(GridInfo)) + 2 * al256(sizeof(uint32_t) * (size_t)n_points) +
-           2 * al256(sizeof(uint32_t) * ((size_t)B + 1)) + al256(sizeof(int64_t));
+    return al256(sizeof(GridInfo)) + 2 * al256(sizeof(uint32_t) * ((size_t)B + 1)) +
+           2 * al256(sizeof(uint32_t) * (size_t)n_points) + al256(sizeof(float4) * (size_t)n_points) +
+           al256(sizeof(unsigned long long) * kScanBlocks);
 }
 
 int cgs_points_to_gaussians(const float *params, const float *m, const float *v, int64_t n, int32_t sh_degree,
@@ -488,42 +779,68 @@ int cgs_points_to_gaussians(const float *params, const float *m, const float *v,
     if (n_points > 0 && (!xyz || !rgb || !workspace)) return CGS_ERR_ARG;
     if (!(init_opacity > 0.f && init_opacity < 1.f)) return CGS_ERR_ARG;
     if (grid_cell_budget(n_points) + 1 >= ((int64_t)1 << 32)) return CGS_ERR_ARG;
-    const int K = (sh_degree + 1) * (sh_degree + 1);
     const int64_t n_out = n + n_points;
+    const int widths[6] = {3, 3, 4, 1, 3, 3 * ((sh_degree + 1) * (sh_degree + 1) - 1)};
+    const float logit = logf(init_opacity / (1.f - init_opacity));
     cudaStream_t s = (cudaStream_t)stream;
-    const int64_t big = n > n_points ? n : n_points;
-    const int blocks = (int)((big + 255) / 256 < 4096 ? (big + 255) / 256 : 4096);
-    if (n > 0) k_copy_prefix<<<blocks, 256, 0, s>>>(params, m, v, n, K, n_out, params_out, m_out, v_out);
+    Runs R{};
+    float *out[3] = {params_out, m_out, v_out};
+    const float *in[3] = {params, m, v};
+    for (int k = 0; k < 3; k++) {
+        int64_t oi = 0, oo = 0;
+        for (int gi = 0; gi < 6; gi++) {
+            const int64_t w = widths[gi];
+            if (n > 0) add_run(R, out[k] + oo, in[k] + oi, w * n, kRunCopy);
+            float *tail = out[k] + oo + w * n;
+            const int64_t len = w * n_points;
+            if (k > 0 || gi == 5)
+                add_run(R, tail, nullptr, len, kRunFill);   // moments and higher bands start at zero
+            else if (gi == 0)
+                add_run(R, tail, xyz, len, kRunCopy);
+            else if (gi == 2)
+                add_run(R, tail, nullptr, len, kRunQuat);
+            else if (gi == 3)
+                add_run(R, tail, nullptr, len, kRunFill, logit);
+            else if (gi == 4)
+                add_run(R, tail, rgb, len, kRunColor);
+            oi += w * n;
+            oo += w * n_out;
+        }
+    }
+    if (n_points > 0 && ((uintptr_t)workspace & 255) != 0) return CGS_ERR_ARG;
+    if (n_points > 0 && workspace_bytes < cgs_points_workspace(n_points)) return CGS_ERR_WORKSPACE;
+    if (R.blocks >= (int64_t)1 << 31) return CGS_ERR_ARG;
+    k_runs<<<(unsigned)R.blocks, kRunThreads, 0, s>>>(R);
     if (n_points == 0) return st_of(cudaGetLastError());
-    if (((uintptr_t)workspace & 255) != 0) return CGS_ERR_ARG;
-    if (workspace_bytes < cgs_points_workspace(n_points)) return CGS_ERR_WORKSPACE;
     const int64_t B = grid_cell_budget(n_points);
     char *w = static_cast<char *>(workspace);
     GridInfo *gi = reinterpret_cast<GridInfo *>(w);
     w += al256(sizeof(GridInfo));
-    uint32_t *cell_of = reinterpret_cast<uint32_t *>(w);
-    w += al256(sizeof(uint32_t) * n_points);
-    uint32_t *ids = reinterpret_cast<uint32_t *>(w);
-    w += al256(sizeof(uint32_t) * n_points);
-    uint32_t *count = reinterpret_cast<uint32_t *>(w);
+    uint32_t *count = reinterpret_cast<uint32_t *>(w);   // next to gi: one memset clears both
     w += al256(sizeof(uint32_t) * (B + 1));
     uint32_t *off = reinterpret_cast<uint32_t *>(w);
     w += al256(sizeof(uint32_t) * (B + 1));
-    int64_t *total = reinterpret_cast<int64_t *>(w);
-    cudaError_t e = cudaMemsetAsync(gi, 0, sizeof(GridInfo), s);
-    if (e == cudaSuccess) e = cudaMemsetAsync(gi->box, 0xff, 3 * sizeof(uint32_t), s);   // minima start high
-    if (e == cudaSuccess) e = cudaMemsetAsync(count, 0, sizeof(uint32_t) * (B + 1), s);
+    uint32_t *cell_of = reinterpret_cast<uint32_t *>(w);   // later the list of far points
+    w += al256(sizeof(uint32_t) * n_points);
+    uint32_t *rank = reinterpret_cast<uint32_t *>(w);
+    w += al256(sizeof(uint32_t) * n_points);
+    float4 *pts = reinterpret_cast<float4 *>(w);
+    w += al256(sizeof(float4) * n_points);
+    unsigned long long *part = reinterpret_cast<unsigned long long *>(w);
+    const cudaError_t e = cudaMemsetAsync(gi, 0, al256(sizeof(GridInfo)) + sizeof(uint32_t) * (B + 1), s);
     if (e != cudaSuccess) return st_of(e);
-    const float logit = logf(init_opacity / (1.f - init_opacity));
     const int pb = (int)((n_points + 255) / 256 < 1024 ? (n_points + 255) / 256 : 1024);
-    k_bbox<<<pb, 256, 0, s>>>(xyz, n_points, gi, status_dev);
-    k_grid_setup<<<1, 32, 0, s>>>(gi, n_points, B);
-    k_cell_count<<<pb, 256, 0, s>>>(xyz, n_points, gi, cell_of, count);
-    k_count_scan<<<1, 1024, 0, s>>>(count, B, off, total);
-    k_cell_scatter<<<pb, 256, 0, s>>>(n_points, cell_of, off, count, ids);
+    k_bbox<<<pb < 304 ? pb : 304, 256, 0, s>>>(xyz, n_points, B, gi, status_dev);
+    k_cell_count<<<pb, 256, 0, s>>>(xyz, n_points, gi, cell_of, rank, count);
+    const int64_t span = scan_span(B);
+    const int sb = scan_blocks(B);
+    k_span_totals<<<sb, kScanThreads, 0, s>>>(count, B, span, part);
+    k_span_scan<<<sb, kScanThreads, 0, s>>>(CountEntry{count}, B, span, part, off, nullptr);
+    k_cell_scatter<<<pb, 256, 0, s>>>(xyz, n_points, cell_of, rank, off, pts);
     const int kb = (int)((n_points + 127) / 128 < 8192 ? (n_points + 127) / 128 : 8192);
-    k_knn_init<<<kb, 128, 0, s>>>(xyz, rgb, n_points, gi, cell_of, off, ids, K, logit, n, n_out, params_out);
-    k_zero_tail<<<pb, 256, 0, s>>>(n, K, n_out, m_out, v_out);
+    float *ls = params_out + 3 * n_out + 3 * n;   // log-scales of the new Gaussians
+    k_knn<<<kb, 128, 0, s>>>(pts, n_points, gi, off, cell_of, ls);
+    k_knn_far<<<304, kFarThreads, 0, s>>>(pts, n_points, gi, off, cell_of, ls);
     return st_of(cudaGetLastError());
 }
 
