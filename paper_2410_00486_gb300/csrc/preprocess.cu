@@ -14,13 +14,11 @@ namespace cgs {
 
 constexpr int kGB = 128;         // Gaussians per block (64: backward 0.53 ms, 128: 0.44 on the 16-view window)
 constexpr int kPreThreads = 256;
-// Resident blocks per SM the backward is compiled for.  With the covariance staged per
-// Gaussian and its chain to scale and rotation run once per Gaussian, three blocks fit
-// (at most 85 registers, 73 KB of shared memory on 16 views): 0.404 -> 0.382 ms on the
-// 16-view window (two blocks at 124 registers before: 0.415 ms).
+// Resident blocks per SM the backward is compiled for (at most 85 registers, 61 KB of shared
+// memory on 16 views).
 constexpr int kPreBwdMinBlocks = 3;
-constexpr int kViewChunk = 64;        // views per compaction round of the backward
-static_assert(kGB * kViewChunk / kPreThreads <= 32, "a thread's visibility bits of a view chunk fit one word");
+constexpr int kViewChunk = 32;   // views whose visibility the backward holds at a time (one word a Gaussian)
+static_assert(kPreThreads == 2 * kGB, "the backward gives a Gaussian two threads");
 constexpr int kCamF = 23;        // staged camera: 20 ABI floats + camera centre
 
 // Real SH normalisation constants (closed forms: sqrt((2l+1)/(4 pi) (l-m)!/(l+m)!) x
@@ -134,9 +132,7 @@ __device__ __forceinline__ void gauss_frame(const Staged &st, int gl, float s[3]
         for (int j = 0; j < 3; j++) M[3 * r + j] = R[3 * r + j] * s[j];
 }
 
-template <int DEG>
 struct Proj {
-    static constexpr int K = (DEG + 1) * (DEG + 1);
     bool visible;
     float t[3], itz;
     float S[6];  // 3-D covariance (staged): xx xy xz yy yz zz
@@ -146,19 +142,26 @@ struct Proj {
     float a, b, c, A, B, C;
     float u, v;
     int radius;
-    float dir[3], dinv;
-    float Y[K];
-    float rgb[3];
-    int mask;
     float o;
 };
 
-// Forward projection of Gaussian gl (block-local) into the staged camera `cam`.
+// Colour of a Gaussian seen from a camera.
 template <int DEG>
+struct Color {
+    static constexpr int K = (DEG + 1) * (DEG + 1);
+    float dir[3], dinv;
+    float Y[K];
+    float rgb[3];
+    int mask;   // channels clamped at 0
+};
+
+// Forward projection of Gaussian gl (block-local) into the staged camera `cam`: centre,
+// depth, conic and opacity, with the radius and the test against the image unless the slot
+// is known to be visible.
+template <bool KNOWN_VISIBLE>
 __device__ __forceinline__ void project(const Staged &st, int gl, const float *cam, const Grid &grid,
-                                        float near_z, Proj<DEG> &o)
+                                        float near_z, Proj &o)
 {
-    constexpr int K = (DEG + 1) * (DEG + 1);
     const float *p = st.means + 3 * gl;
     const float *Rc = cam;
     o.visible = false;
@@ -205,6 +208,9 @@ __device__ __forceinline__ void project(const Staged &st, int gl, const float *c
     o.A = o.c * idet;
     o.B = -o.b * idet;
     o.C = o.a * idet;
+    o.o = 1.0f / (1.0f + expf(-st.opac[gl]));
+    o.visible = true;
+    if (KNOWN_VISIBLE) return;
     // largest eigenvalue; mid^2 - det written as ((a - c)/2)^2 + b^2 (no cancellation)
     float hd = 0.5f * (o.a - o.c);
     float disc = hd * hd + o.b * o.b;
@@ -216,10 +222,16 @@ __device__ __forceinline__ void project(const Staged &st, int gl, const float *c
     Rect rc = tile_rect(o.u, o.v, o.radius, grid);
     if (rc.x1 <= rc.x0 || rc.y1 <= rc.y0) {
         o.radius = 0;
-        return;
+        o.visible = false;
     }
+}
 
-    // colour from SH at the direction camera centre -> mean
+// Colour from SH at the direction camera centre -> mean.
+template <int DEG>
+__device__ __forceinline__ void color(const Staged &st, int gl, const float *cam, Color<DEG> &o)
+{
+    constexpr int K = (DEG + 1) * (DEG + 1);
+    const float *p = st.means + 3 * gl;
     float d0 = p[0] - cam[20], d1 = p[1] - cam[21], d2 = p[2] - cam[22];
     float dn = sqrtf(d0 * d0 + d1 * d1 + d2 * d2);
     o.dinv = 1.0f / dn;
@@ -240,11 +252,22 @@ __device__ __forceinline__ void project(const Staged &st, int gl, const float *c
         }
         o.rgb[ch] = acc;
     }
-    o.o = 1.0f / (1.0f + expf(-st.opac[gl]));
-    o.visible = true;
 }
 
-// Stage the block's parameter slices and the cameras into shared memory.
+__device__ __forceinline__ void async_copy(float *dst, const float *src, bool wide)
+{
+    const uint32_t d = (uint32_t)__cvta_generic_to_shared(dst);
+    if (wide)
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d), "l"(src) : "memory");
+    else
+        asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(d), "l"(src) : "memory");
+}
+
+// Stage the block's parameter slices and the cameras into shared memory.  Every copy is
+// asynchronous, so the whole slice is in flight at once without a register; where the group
+// starts are 16-byte aligned (n a multiple of four) they move 16 bytes each.  Four loads
+// before their four stores left a block several memory latencies: with one view of 100k
+// Gaussians, where staging is most of the work, the projection takes 8.1 us after 16.1.
 template <int DEG>
 __device__ __forceinline__ Staged stage(float *sm, const float *__restrict__ P, int64_t n, int64_t g0,
                                         int cnt, const cgs_camera *__restrict__ cams, int V)
@@ -263,24 +286,10 @@ __device__ __forceinline__ Staged stage(float *sm, const float *__restrict__ P, 
             continue;
         }
         const float *src = P + offs[gi] + (int64_t)w * g0;
-        // four loads in flight before their stores: one load and store at a time left each
-        // block waiting a memory latency per element it staged (on the 16-view window:
-        // backward 0.388 -> 0.337 ms, projection 0.166 -> 0.139 ms; 2, 3, 8 and 16 measured
-        // slower)
         const int tot = w * cnt;
-        for (int i0 = threadIdx.x; i0 < tot; i0 += 4 * blockDim.x) {
-            float x[4];
-#pragma unroll
-            for (int k = 0; k < 4; k++) {
-                const int i = i0 + k * (int)blockDim.x;
-                x[k] = i < tot ? __ldg(src + i) : 0.f;
-            }
-#pragma unroll
-            for (int k = 0; k < 4; k++) {
-                const int i = i0 + k * (int)blockDim.x;
-                if (i < tot) cur[i] = x[k];
-            }
-        }
+        const int quads = ((uintptr_t)src & 15) == 0 ? tot / 4 : 0;   // cur is 16-byte aligned: kGB is
+        for (int i = threadIdx.x; i < quads; i += blockDim.x) async_copy(cur + 4 * i, src + 4 * i, true);
+        for (int i = 4 * quads + (int)threadIdx.x; i < tot; i += blockDim.x) async_copy(cur + i, src + i, false);
         *dst[gi] = cur;
         cur += w * kGB;
     }
@@ -289,6 +298,7 @@ __device__ __forceinline__ Staged stage(float *sm, const float *__restrict__ P, 
     // cameras: 20 ABI floats + centre c = -R^T t
     const float *cf = reinterpret_cast<const float *>(cams);
     for (int i = threadIdx.x; i < V * 20; i += blockDim.x) cur[(i / 20) * kCamF + (i % 20)] = __ldg(cf + i);
+    asm volatile("cp.async.wait_all;" ::: "memory");
     __syncthreads();
     for (int v = threadIdx.x; v < V; v += blockDim.x) {
         float *c = cur + v * kCamF;
@@ -323,7 +333,7 @@ __global__ void __launch_bounds__(kPreThreads)
 k_preprocess(const float *__restrict__ P, int64_t n, const cgs_camera *__restrict__ cams, int V,
              Grid grid, float near_z, float4 *__restrict__ rec, float4 *__restrict__ sgrad)
 {
-    extern __shared__ float sm[];
+    extern __shared__ __align__(16) float sm[];
     const int64_t g0 = (int64_t)blockIdx.x * kGB;
     const int cnt = (int)min((int64_t)kGB, n - g0);
     Staged st = stage<DEG>(sm, P, n, g0, cnt, cams, V);
@@ -331,8 +341,8 @@ k_preprocess(const float *__restrict__ P, int64_t n, const cgs_camera *__restric
         const int gl = it % kGB, v = it / kGB;
         if (gl >= cnt) continue;
         const int64_t slot = (int64_t)v * n + g0 + gl;
-        Proj<DEG> o;
-        project<DEG>(st, gl, st.cams + v * kCamF, grid, near_z, o);
+        Proj o;
+        project<false>(st, gl, st.cams + v * kCamF, grid, near_z, o);
         float4 *r = rec + kRec4 * slot;
         if (!o.visible) {
             // the whole record (radius 0 marks it culled) and slot gradient: with only the
@@ -350,11 +360,13 @@ k_preprocess(const float *__restrict__ P, int64_t n, const cgs_camera *__restric
             }
             continue;
         }
+        Color<DEG> col;
+        color<DEG>(st, gl, st.cams + v * kCamF, col);
         r[0] = make_float4(o.u, o.v, o.A, o.B);
         r[1] = make_float4(o.C, o.o, o.t[2], __int_as_float(o.radius));
         // tau = -ln(255 o): alpha >= 1/255 exactly when power >= tau (the tile test and the
         // raster kernels' exponent threshold)
-        r[2] = make_float4(o.rgb[0], o.rgb[1], o.rgb[2], -logf(255.0f * o.o));
+        r[2] = make_float4(col.rgb[0], col.rgb[1], col.rgb[2], -logf(255.0f * o.o));
         if (sgrad) {
             float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
             float4 *gp = sgrad + kRec4 * slot;
@@ -365,42 +377,17 @@ k_preprocess(const float *__restrict__ P, int64_t n, const cgs_camera *__restric
     }
 }
 
-// Backward of one visible slot: accumulates parameter gradients (and dL/dSigma, whose
-// chain to scale and rotation sigma_bwd runs once per Gaussian) into the block's shared
-// accumulators (acc has the staged layout) with shared-memory atomics.
-template <int DEG>
-__device__ __forceinline__ void project_bwd(const Staged &st, int gl, const float *cam, const Proj<DEG> &o,
-                                            float4 G0, float4 G1, float4 G2, float *acc)
+// Backward of one visible slot through the projection, added to the Gaussian's sums acc:
+// mean (3), opacity logit, dL/dSigma (upper triangle, 6).
+__device__ __forceinline__ void project_bwd(const float *cam, const Proj &o, const float4 &G0, const float4 &G1,
+                                            float *acc)
 {
-    constexpr int K = (DEG + 1) * (DEG + 1);
-    float *a_means = acc;   // scales and quaternions get theirs once per Gaussian (sigma_bwd)
-    float *a_opac = acc + 10 * kGB;
-    float *a_dc = acc + 11 * kGB;
-    float *a_rest = acc + 14 * kGB;
     const float *Rc = cam;
     const float fx = cam[12], fy = cam[13];
     const float gu = G0.x, gv = G0.y, gA = G0.z, gB = G0.w, gC = G1.x, go = G1.y, gz = G1.z;
-    float dmean[3] = {0.f, 0.f, 0.f};
-
-    // colour -> SH coefficients and view direction (0 through a clamped channel)
-    float gc[3] = {(o.mask & 1) ? 0.f : G2.x, (o.mask & 2) ? 0.f : G2.y, (o.mask & 4) ? 0.f : G2.z};
-    for (int ch = 0; ch < 3; ch++) atomicAdd(&a_dc[3 * gl + ch], o.Y[0] * gc[ch]);
-    if (DEG > 0) {
-        const float *rest = st.rest + 3 * (K - 1) * gl;
-        float wk[K];
-        wk[0] = 0.f;
-        for (int k = 1; k < K; k++) {
-            wk[k] = rest[3 * (k - 1)] * gc[0] + rest[3 * (k - 1) + 1] * gc[1] + rest[3 * (k - 1) + 2] * gc[2];
-            for (int ch = 0; ch < 3; ch++) atomicAdd(&a_rest[3 * (K - 1) * gl + 3 * (k - 1) + ch], o.Y[k] * gc[ch]);
-        }
-        float ddir[3] = {0.f, 0.f, 0.f};
-        sh_basis_vjp<DEG>(o.dir[0], o.dir[1], o.dir[2], wk, ddir);
-        float dd = ddir[0] * o.dir[0] + ddir[1] * o.dir[1] + ddir[2] * o.dir[2];
-        for (int i = 0; i < 3; i++) dmean[i] += (ddir[i] - o.dir[i] * dd) * o.dinv;
-    }
 
     // opacity logit
-    atomicAdd(&a_opac[gl], go * o.o * (1.f - o.o));
+    acc[3] += go * o.o * (1.f - o.o);
 
     // conic Q = Sigma'^-1:  dL/dSigma' = -Q G_Q Q,  G_Q = [[gA, gB/2], [gB/2, gC]]
     const float hB = 0.5f * gB;
@@ -454,33 +441,54 @@ __device__ __forceinline__ void project_bwd(const Staged &st, int gl, const floa
     dt1 += gv * fy * itz;
     dt2 -= gv * fy * o.t[1] * itz2;
     dt2 += gz;
-    for (int i = 0; i < 3; i++) dmean[i] += Rc[i] * dt0 + Rc[3 + i] * dt1 + Rc[6 + i] * dt2;
-    for (int i = 0; i < 3; i++) atomicAdd(&a_means[3 * gl + i], dmean[i]);
+    for (int i = 0; i < 3; i++) acc[i] += Rc[i] * dt0 + Rc[3 + i] * dt1 + Rc[6 + i] * dt2;
 
-    // dL/dSigma (symmetric; upper triangle) gathered over the Gaussian's views: the chain to
-    // scale and rotation is linear in it and runs once per Gaussian (sigma_bwd)
-    float *a_cov = acc + (14 + 3 * (K - 1)) * kGB;
-    atomicAdd(&a_cov[6 * gl + 0], GS[0]);
-    atomicAdd(&a_cov[6 * gl + 1], GS[1]);
-    atomicAdd(&a_cov[6 * gl + 2], GS[2]);
-    atomicAdd(&a_cov[6 * gl + 3], GS[4]);
-    atomicAdd(&a_cov[6 * gl + 4], GS[5]);
-    atomicAdd(&a_cov[6 * gl + 5], GS[8]);
+    // dL/dSigma (symmetric; upper triangle): the chain to scale and rotation is linear in it
+    // and runs once per Gaussian (sigma_bwd)
+    acc[4] += GS[0];
+    acc[5] += GS[1];
+    acc[6] += GS[2];
+    acc[7] += GS[4];
+    acc[8] += GS[5];
+    acc[9] += GS[8];
+}
+
+// Backward of one visible slot through its colour (0 through a clamped channel): SH
+// coefficients, added to this thread's dc and rest rows, and the mean by the view direction.
+template <int DEG>
+__device__ __forceinline__ void color_bwd(const Staged &st, int gl, const float *cam, const float4 &G2,
+                                          float dc[3], float *rest_acc, float dmean[3])
+{
+    constexpr int K = (DEG + 1) * (DEG + 1);
+    Color<DEG> o;
+    color<DEG>(st, gl, cam, o);
+    asm volatile("" ::: "memory");   // the rest row is read again below, not held in registers meanwhile
+    const float gc[3] = {(o.mask & 1) ? 0.f : G2.x, (o.mask & 2) ? 0.f : G2.y, (o.mask & 4) ? 0.f : G2.z};
+    for (int ch = 0; ch < 3; ch++) dc[ch] += o.Y[0] * gc[ch];
+    if (DEG > 0) {
+        const float *rest = st.rest + 3 * (K - 1) * gl;
+        float wk[K];
+        wk[0] = 0.f;
+#pragma unroll
+        for (int k = 1; k < K; k++) {
+            wk[k] = rest[3 * (k - 1)] * gc[0] + rest[3 * (k - 1) + 1] * gc[1] + rest[3 * (k - 1) + 2] * gc[2];
+#pragma unroll
+            for (int ch = 0; ch < 3; ch++) rest_acc[3 * (k - 1) + ch] += o.Y[k] * gc[ch];
+        }
+        float ddir[3] = {0.f, 0.f, 0.f};
+        sh_basis_vjp<DEG>(o.dir[0], o.dir[1], o.dir[2], wk, ddir);
+        float dd = ddir[0] * o.dir[0] + ddir[1] * o.dir[1] + ddir[2] * o.dir[2];
+        for (int i = 0; i < 3; i++) dmean[i] += (ddir[i] - o.dir[i] * dd) * o.dinv;
+    }
 }
 
 // Sigma = M M^T, M = R diag(s), with G = dL/dSigma summed over the views: dL/dM = 2 G M,
 // then dL/ds and dL/dR, and the rotation of the unit quaternion back through its
-// normalisation; written into the scale and quaternion accumulators of Gaussian gl.
-template <int DEG>
-__device__ __forceinline__ void sigma_bwd(const Staged &st, int gl, float *acc)
+// normalisation.
+__device__ __forceinline__ void sigma_bwd(const Staged &st, int gl, const float g6[6], float scales[3], float quat[4])
 {
-    constexpr int K = (DEG + 1) * (DEG + 1);
-    float *a_scales = acc + 3 * kGB;
-    float *a_quats = acc + 6 * kGB;
-    const float *a_cov = acc + (14 + 3 * (K - 1)) * kGB;
     float sc[3], qn[4], qinv, R[9], M[9];
     gauss_frame(st, gl, sc, qn, qinv, R, M);
-    const float *g6 = a_cov + 6 * gl;
     const float GS[9] = {g6[0], g6[1], g6[2], g6[1], g6[3], g6[4], g6[2], g6[4], g6[5]};
     float GR[9];
     for (int j = 0; j < 3; j++) {
@@ -490,7 +498,7 @@ __device__ __forceinline__ void sigma_bwd(const Staged &st, int gl, float *acc)
             ds += gm * R[3 * r + j];
             GR[3 * r + j] = gm * sc[j];
         }
-        a_scales[3 * gl + j] = ds * sc[j];
+        scales[j] = ds * sc[j];
     }
     const float w = qn[0], x = qn[1], y = qn[2], z = qn[3];
     float dq0 = 2.f * (-z * GR[1] + y * GR[2] + z * GR[3] - x * GR[5] - y * GR[6] + x * GR[7]);
@@ -501,12 +509,20 @@ __device__ __forceinline__ void sigma_bwd(const Staged &st, int gl, float *acc)
     float dq3 = 2.f * (-2.f * z * GR[0] - w * GR[1] + x * GR[2] + w * GR[3] - 2.f * z * GR[4] + y * GR[5] +
                        x * GR[6] + y * GR[7]);
     float pr = dq0 * w + dq1 * x + dq2 * y + dq3 * z;
-    a_quats[4 * gl + 0] = (dq0 - w * pr) * qinv;
-    a_quats[4 * gl + 1] = (dq1 - x * pr) * qinv;
-    a_quats[4 * gl + 2] = (dq2 - y * pr) * qinv;
-    a_quats[4 * gl + 3] = (dq3 - z * pr) * qinv;
+    quat[0] = (dq0 - w * pr) * qinv;
+    quat[1] = (dq1 - x * pr) * qinv;
+    quat[2] = (dq2 - y * pr) * qinv;
+    quat[3] = (dq3 - z * pr) * qinv;
 }
 
+// A Gaussian has two threads, a block's first half for the geometry and its second half for
+// the colours: each walks the Gaussian's visible views in order and gathers its sums in
+// registers (the SH rows, too many for them, in this thread's row of shared memory), so no
+// two threads add to one word.  The lanes of a warp wait for the one with the most views,
+// which costs less than 58 shared-memory float atomics a slot (loops of compare-and-swap) on
+// compacted slots did: 281 us after 332 on 16 views of 300k Gaussians, 130 after 142 on 8 of
+// 200k, 20.5 after 35.2 on one of 100k.  Bound by the chain rule's arithmetic and, with one
+// view, by HBM.
 template <int DEG>
 __global__ void __launch_bounds__(kPreThreads, kPreBwdMinBlocks)
 k_preprocess_bwd(const float *__restrict__ P, int64_t n, const cgs_camera *__restrict__ cams, int V,
@@ -515,92 +531,117 @@ k_preprocess_bwd(const float *__restrict__ P, int64_t n, const cgs_camera *__res
                  float *__restrict__ denom, float *__restrict__ max_r2d)
 {
     constexpr int K = (DEG + 1) * (DEG + 1);
-    constexpr int NS = staged_floats<DEG>();
-    extern __shared__ float sm[];
+    constexpr int R3 = 3 * (K - 1);
+    extern __shared__ __align__(16) float sm[];
     const int64_t g0 = (int64_t)blockIdx.x * kGB;
     const int cnt = (int)min((int64_t)kGB, n - g0);
-    float *acc = sm;                    // gradient accumulators, staged layout
-    float *dstat = sm + NS;             // densify stats: accum, denom, max radius (3 x kGB)
-    for (int i = threadIdx.x; i < NS + 3 * kGB; i += blockDim.x) acc[i] = 0.f;
-    // visible (view, Gaussian) items of the block, compacted (per chunk of kViewChunk views)
-    // so that the chain rule runs with full warps: most slots of a view are culled
-    uint16_t *items = reinterpret_cast<uint16_t *>(sm + 2 * NS + 3 * kGB + V * kCamF);
-    __shared__ int wcount[kPreThreads / 32];
-    Staged st = stage<DEG>(sm + NS + 3 * kGB, P, n, g0, cnt, cams, V);
-    const bool stats = accum != nullptr;
-    const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
+    // SH gradients (dc, then rest, as in the output), the mean's gradient by the view
+    // directions, and the largest radius a thread saw
+    float *shg = sm, *sdm = shg + (3 + R3) * kGB, *srad = sdm + 3 * kGB;
+    __shared__ uint32_t smask[2][kGB];   // visible views of the chunk, 16 a thread
+    for (int i = threadIdx.x; i < R3 * kGB; i += kPreThreads) shg[3 * kGB + i] = 0.f;
+    Staged st = stage<DEG>(srad + kGB, P, n, g0, cnt, cams, V);
+    const int gl = threadIdx.x % kGB;
+    const bool geometry = threadIdx.x < kGB;   // warp-uniform
+    const int64_t slot0 = g0 + gl;
+    // geometry: mean (3), opacity, dL/dSigma (6), view-space gradient norms, views seen;
+    // colour: dc (3), mean (3)
+    float acc[12];
+#pragma unroll
+    for (int i = 0; i < 12; i++) acc[i] = 0.f;
+    int rmax = 0;
     for (int v0 = 0; v0 < V; v0 += kViewChunk) {
-        const int nit = kGB * min(kViewChunk, V - v0);
-        int nitems = 0;
-        // visibility of this thread's items of the chunk, all loads in flight together
-        // (one bit per round of kPreThreads items)
-        uint32_t vismask = 0;
-#pragma unroll 8
-        for (int c0 = 0, rb = 0; c0 < nit; c0 += kPreThreads, rb++) {
-            const int it = c0 + (int)threadIdx.x;
-            const int gl = it % kGB, v = v0 + it / kGB;
-            if (it < nit && gl < cnt) {
-                const float *r = reinterpret_cast<const float *>(rec + kRec4 * ((int64_t)v * n + g0 + gl));
-                if (__float_as_int(__ldg(r + 7)) > 0) vismask |= 1u << rb;
+        uint32_t vis = 0u;
+        const int h0 = v0 + (geometry ? 0 : kViewChunk / 2);
+        if (gl < cnt) {
+#pragma unroll
+            for (int k = 0; k < kViewChunk / 2; k++) {   // all loads in flight together
+                if (h0 + k >= V) break;
+                const float *r = reinterpret_cast<const float *>(rec + kRec4 * ((int64_t)(h0 + k) * n + slot0));
+                const int rad = __float_as_int(__ldg(r + 7));
+                if (rad > 0) vis |= 1u << k;
+                rmax = max(rmax, rad);
             }
         }
-        for (int c0 = 0, rb = 0; c0 < nit; c0 += kPreThreads, rb++) {
-            const int it = c0 + (int)threadIdx.x;
-            const bool vis = (vismask >> rb) & 1u;
-            const unsigned b = __ballot_sync(kFull, vis);
-            if (lane == 0) wcount[wp] = __popc(b);
-            __syncthreads();
-            int off = nitems, tot = 0;
-            for (int i = 0; i < kPreThreads / 32; i++) {
-                off += i < wp ? wcount[i] : 0;
-                tot += wcount[i];
-            }
-            if (vis) items[off + __popc(b & ((1u << lane) - 1u))] = (uint16_t)it;
-            nitems += tot;
-            __syncthreads();
+        __syncthreads();   // the previous chunk's words have been read
+        smask[geometry ? 0 : 1][gl] = vis;
+        __syncthreads();
+        uint32_t m = smask[0][gl] | (smask[1][gl] << (kViewChunk / 2));
+        // the next slot's gradient is on its way while this one's runs
+        const float4 *gp = sgrad + kRec4 * ((int64_t)v0 * n + slot0) + (geometry ? 0 : 2);
+        const int64_t vstep = kRec4 * n;
+        float4 G0 = make_float4(0.f, 0.f, 0.f, 0.f), G1 = G0;
+        if (m) {
+            G0 = __ldg(gp + (__ffs(m) - 1) * vstep);
+            if (geometry) G1 = __ldg(gp + (__ffs(m) - 1) * vstep + 1);
         }
-        for (int k = threadIdx.x; k < nitems; k += blockDim.x) {
-            const int it = items[k];
-            const int gl = it % kGB, v = v0 + it / kGB;
-            const int64_t slot = (int64_t)v * n + g0 + gl;
-            const float4 *r = rec + kRec4 * slot;
-            const int rad = __float_as_int(__ldg(reinterpret_cast<const float *>(r) + 7));
-            const float4 *gp = sgrad + kRec4 * slot;
-            float4 G0 = gp[0], G1 = gp[1], G2 = gp[2];
-            Proj<DEG> o;
-            project<DEG>(st, gl, st.cams + v * kCamF, grid, near_z, o);
-            if (!o.visible) continue;   // cannot happen for a slot the forward marked visible
-            project_bwd<DEG>(st, gl, st.cams + v * kCamF, o, G0, G1, G2, acc);
-            if (stats) {
-                float gx = G0.x * 0.5f * (float)grid.W, gy = G0.y * 0.5f * (float)grid.H;
-                atomicAdd(&dstat[gl], sqrtf(gx * gx + gy * gy));
-                atomicAdd(&dstat[kGB + gl], 1.0f);
-                atomicMax(reinterpret_cast<int *>(&dstat[2 * kGB + gl]), __float_as_int((float)rad));
+        while (m) {
+            const float *cam = st.cams + (v0 + __ffs(m) - 1) * kCamF;
+            const float4 C0 = G0, C1 = G1;
+            m &= m - 1u;
+            if (m) {
+                G0 = __ldg(gp + (__ffs(m) - 1) * vstep);
+                if (geometry) G1 = __ldg(gp + (__ffs(m) - 1) * vstep + 1);
+            }
+            if (geometry) {
+                Proj o;
+                project<true>(st, gl, cam, grid, near_z, o);
+                if (!o.visible) continue;   // cannot happen for a slot the forward marked visible
+                project_bwd(cam, o, C0, C1, acc);
+                const float gx = C0.x * 0.5f * (float)grid.W, gy = C0.y * 0.5f * (float)grid.H;
+                acc[10] += sqrtf(gx * gx + gy * gy);
+                acc[11] += 1.f;
+            } else {
+                color_bwd<DEG>(st, gl, cam, C0, acc, shg + 3 * kGB + R3 * gl, acc + 3);
             }
         }
-        __syncthreads();   // the item list is rebuilt for the next chunk of views
     }
-    for (int gl = threadIdx.x; gl < cnt; gl += blockDim.x) sigma_bwd<DEG>(st, gl, acc);
+    if (!geometry) {
+        for (int i = 0; i < 3; i++) {
+            shg[3 * gl + i] = acc[i];
+            sdm[3 * gl + i] = acc[3 + i];
+        }
+        srad[gl] = (float)rmax;
+    }
+    __syncthreads();   // and the parameters have been read by the colour threads
+    if (geometry && gl < cnt) {
+        float ds[3], dq[4];
+        sigma_bwd(st, gl, acc + 4, ds, dq);
+        // the gradients take the place of the thread's own staged parameters
+        float *o = const_cast<float *>(st.means);
+        for (int i = 0; i < 3; i++) o[3 * gl + i] = acc[i] + sdm[3 * gl + i];
+        for (int i = 0; i < 3; i++) o[3 * kGB + 3 * gl + i] = ds[i];
+        for (int i = 0; i < 4; i++) o[6 * kGB + 4 * gl + i] = dq[i];
+        o[10 * kGB + gl] = acc[3];
+        if (accum) {
+            accum[g0 + gl] += acc[10];
+            denom[g0 + gl] += acc[11];
+            max_r2d[g0 + gl] = fmaxf(max_r2d[g0 + gl], fmaxf((float)rmax, srad[gl]));
+        }
+    }
     __syncthreads();
     // write the block's slice of every group (coalesced)
     const Layout L = param_layout(n, DEG);
-    const int widths[6] = {3, 3, 4, 1, 3, 3 * (K - 1)};
+    const int widths[6] = {3, 3, 4, 1, 3, R3};
     const int64_t offs[6] = {L.means, L.scales, L.quats, L.opac, L.dc, L.rest};
-    int soff = 0;
+    const float *from[6] = {st.means, st.means + 3 * kGB, st.means + 6 * kGB, st.means + 10 * kGB, shg, shg + 3 * kGB};
+#pragma unroll
     for (int gi = 0; gi < 6; gi++) {
-        const int w = widths[gi];
+        const int w = widths[gi], tot = w * cnt;
         if (w == 0) continue;
         float *dst = pgrad + offs[gi] + (int64_t)w * g0;
-        const float *src = acc + soff;
-        for (int i = threadIdx.x; i < w * cnt; i += blockDim.x) dst[i] = accumulate ? dst[i] + src[i] : src[i];
-        soff += w * kGB;
-    }
-    if (stats) {
-        for (int i = threadIdx.x; i < cnt; i += blockDim.x) {
-            accum[g0 + i] += dstat[i];
-            denom[g0 + i] += dstat[kGB + i];
-            max_r2d[g0 + i] = fmaxf(max_r2d[g0 + i], dstat[2 * kGB + i]);
+        const float *src = from[gi];
+        const int quads = ((uintptr_t)dst & 15) == 0 ? tot / 4 : 0;
+        for (int i = threadIdx.x; i < quads; i += kPreThreads) {
+            float4 x = reinterpret_cast<const float4 *>(src)[i];
+            if (accumulate) {
+                const float4 y = reinterpret_cast<float4 *>(dst)[i];
+                x = make_float4(y.x + x.x, y.y + x.y, y.z + x.z, y.w + x.w);
+            }
+            reinterpret_cast<float4 *>(dst)[i] = x;
         }
+        for (int i = 4 * quads + (int)threadIdx.x; i < tot; i += kPreThreads)
+            dst[i] = accumulate ? dst[i] + src[i] : src[i];
     }
 }
 
@@ -619,7 +660,8 @@ static cudaError_t launch_pre(const float *P, int64_t n, const cgs_camera *cams,
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     int blocks = (int)((n + kGB - 1) / kGB);
-    k<<<blocks, kPreThreads, smem, s>>>(P, n, cams, V, g, near_z, rec, sgrad);
+    // one view has an item for half of the threads only
+    k<<<blocks, V == 1 ? kGB : kPreThreads, smem, s>>>(P, n, cams, V, g, near_z, rec, sgrad);
     return cudaGetLastError();
 }
 
@@ -628,8 +670,7 @@ static cudaError_t launch_pre_bwd(const float *P, int64_t n, const cgs_camera *c
                                   float near_z, const float4 *rec, const float4 *sgrad, float *pgrad,
                                   int accumulate, float *accum, float *denom, float *maxr, cudaStream_t s)
 {
-    size_t smem = sizeof(float) * (2 * (size_t)staged_floats<DEG>() + 3 * kGB + (size_t)V * kCamF) +
-                  sizeof(uint16_t) * (size_t)kGB * min(V, kViewChunk);
+    size_t smem = pre_smem<DEG>(V) + sizeof(float) * kGB * (3 * (DEG + 1) * (DEG + 1) + 4);
     auto k = k_preprocess_bwd<DEG>;
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
