@@ -39,15 +39,27 @@ constexpr size_t kAggMaxSmem = 96 * 1024;   // per-view tile histogram in shared
 // leave fewer than four blocks per SM.  Measured (whole sort, ms): the 16-view 300k window
 // 0.844 / 0.831 / 0.862 / 1.024 for 1024 / 2048 / 4096 / 8192; one 100k view 0.101 / 0.115 /
 // 0.153 (49 blocks of 2048 slots for 152 SMs).
-constexpr int kChunkLarge = 2048, kChunkSmall = 1024;
+// A small window takes smaller chunks, down to 256, until every SM has a block (one 640x480
+// view of 40k Gaussians: count 12.0 -> 9.9 us, 160x120 of 2k: 7.7 -> 4.8, scatter 6.3 -> 4.3;
+// one 1200x680 view of 100k, in chunks of 512: 25 and 29 us as before).
+constexpr int kChunkLarge = 2048, kChunkSmall = 1024, kChunkMin = 256;
 static int chunk_for(int64_t n, int64_t V, int num_sms)
 {
-    return (n + kChunkLarge - 1) / kChunkLarge * V >= 4 * (int64_t)num_sms ? kChunkLarge : kChunkSmall;
+    auto blocks = [&](int chunk) { return (n + chunk - 1) / chunk * V; };
+    if (blocks(kChunkLarge) >= 4 * (int64_t)num_sms) return kChunkLarge;
+    int chunk = kChunkSmall;
+    while (chunk > kChunkMin && blocks(chunk) < num_sms) chunk /= 2;
+    return chunk;
 }
 
 // Scan of the per-tile counts: blocks of kScanThreads threads, kScanPer entries each.
 constexpr int kScanThreads = 1024, kScanPer = 4, kScanSpan = kScanThreads * kScanPer;
-constexpr int kLenBuckets = 33;   // list-length buckets of the work order: 0 (empty), 1 + floor(log2 len)
+// List-length buckets of the work order: lengths below 8 by themselves, then eight to the
+// octave (len_bucket).  The raster kernels take the longest lists first, and with one bucket
+// to the octave lists of up to twice another's length came in any order: the 8-view 200k
+// window's iteration took 1341 us, with eight 1260, four views' render 507 and 485.
+constexpr int kLenBuckets = 240;
+static_assert(kLenBuckets <= 256, "the scan forms the bucket suffix sums with eight warps");
 
 struct BinWs {
     uint32_t *count;     // [Ttot + 1]
@@ -395,10 +407,15 @@ k_count_agg(const float4 *__restrict__ rec, int64_t n, int chunk, Grid g, uint32
 }
 
 // Multi-block scan of the per-tile counts and the raster work order (tiles by
-// decreasing list length, bucketed by floor(log2(len)), longest bucket first; tile order
-// inside a bucket is arbitrary), in two launches over blocks of kScanSpan tiles.
+// decreasing list length, in buckets of an eighth of an octave, longest bucket first; tile
+// order inside a bucket is arbitrary), in two launches over blocks of kScanSpan tiles.
 // k_scan_part: each block's instance total and its histogram of length buckets.
-__device__ __forceinline__ uint32_t len_bucket(uint32_t len) { return len ? 32 - __clz(len) : 0; }
+__device__ __forceinline__ uint32_t len_bucket(uint32_t len)
+{
+    if (len < 8u) return len;
+    const int e = 31 - __clz(len);
+    return 8u * (uint32_t)(e - 2) + ((len >> (e - 3)) & 7u);
+}
 
 __global__ void __launch_bounds__(kScanThreads)
 k_scan_part(const uint32_t *__restrict__ count, int64_t Ttot, unsigned long long *__restrict__ part,
@@ -434,7 +451,13 @@ k_scan_part(const uint32_t *__restrict__ count, int64_t Ttot, unsigned long long
 // starts (written over the counts, for the scatter) and ranges, both clamped to the
 // capacity, and places its tiles in the work order after every longer bucket's tiles and
 // the earlier blocks' tiles of the same bucket.  Block 0 writes the instance total, the
-// capacity status, and clears the long-tile list.
+// capacity status, and clears the long-tile list.  With ONE (a window of one block of
+// tiles, as a single view has) it forms the totals and the histogram itself and
+// k_scan_part is not launched.  Tiles of the same length bucket in a warp take their
+// places with one atomic: a bucket holds a large share of the tiles, and their atomics on
+// its one word queue (one 1200x680 view: 14.6 us in two launches, 8 in one with 240 buckets;
+// 160x120: 11.7 and 4.3).
+template <bool ONE>
 __global__ void __launch_bounds__(kScanThreads)
 k_scan_out(uint32_t *__restrict__ count, int64_t Ttot, int64_t capacity, const unsigned long long *__restrict__ part,
            const uint32_t *__restrict__ bhist, int nblocks, uint32_t *__restrict__ ranges,
@@ -443,79 +466,119 @@ k_scan_out(uint32_t *__restrict__ count, int64_t Ttot, int64_t capacity, const u
 {
     __shared__ unsigned long long wtot[kScanThreads / 32];
     __shared__ unsigned long long s_pre;
-    __shared__ uint32_t btot[kLenBuckets], offs[kLenBuckets];
+    __shared__ uint32_t btot[kLenBuckets], offs[kLenBuckets], blong[8];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const unsigned long long cap = (unsigned long long)capacity;
-    if (threadIdx.x == 0) {
-        unsigned long long pre = 0, tot = 0;
-        for (int b = 0; b < nblocks; b++) {
-            const unsigned long long x = part[b];
-            pre += b < (int)blockIdx.x ? x : 0ull;
-            tot += x;
-        }
-        s_pre = pre;
-        if (blockIdx.x == 0) {
-            *nbig = 0u;   // the long-tile list of k_sort_tiles starts empty
-            *n_inst = (int64_t)tot;
-            count[Ttot] = (uint32_t)min(tot, cap);
-            if (tot > cap) set_status(status, CGS_ERR_CAPACITY);
-        }
+    // the thread's kScanPer consecutive tiles, and their peers in the warp by length bucket
+    const int64_t t0 = (int64_t)blockIdx.x * kScanSpan + kScanPer * (int64_t)threadIdx.x;
+    uint32_t c[kScanPer], peers[kScanPer];
+    unsigned long long tsum = 0;
+#pragma unroll
+    for (int k = 0; k < kScanPer; k++) {
+        c[k] = t0 + k < Ttot ? count[t0 + k] : 0u;
+        tsum += c[k];
     }
-    if (order && threadIdx.x < kLenBuckets) {
+    if (order) {   // tiles past the end share the key no bucket has
+#pragma unroll
+        for (int k = 0; k < kScanPer; k++)
+            peers[k] = __match_any_sync(kFull, t0 + k < Ttot ? len_bucket(c[k]) : 255u);
+    }
+    if (threadIdx.x < kLenBuckets) {
         uint32_t all = 0, before = 0;
-        for (int b = 0; b < nblocks; b++) {
-            const uint32_t x = bhist[(int64_t)b * kLenBuckets + threadIdx.x];
-            all += x;
-            before += b < (int)blockIdx.x ? x : 0u;
+        if (!ONE && order) {
+#pragma unroll 4
+            for (int b = 0; b < nblocks; b++) {
+                const uint32_t x = bhist[(int64_t)b * kLenBuckets + threadIdx.x];
+                all += x;
+                before += b < (int)blockIdx.x ? x : 0u;
+            }
         }
         btot[threadIdx.x] = all;
         offs[threadIdx.x] = before;
     }
+    unsigned long long incl = tsum;
+#pragma unroll
+    for (int off = 1; off < 32; off <<= 1) {
+        const unsigned long long y = __shfl_up_sync(kFull, incl, off);
+        if (lane >= off) incl += y;
+    }
+    if (lane == 31) wtot[w] = incl;
+    if (!ONE && w == kScanThreads / 32 - 1) {   // totals of the other blocks
+        unsigned long long pre = 0, tot = 0;
+        for (int b = lane; b < nblocks; b += 32) {
+            const unsigned long long x = part[b];
+            pre += b < (int)blockIdx.x ? x : 0ull;
+            tot += x;
+        }
+        for (int off = 16; off > 0; off >>= 1) {
+            pre += __shfl_xor_sync(kFull, pre, off);
+            tot += __shfl_xor_sync(kFull, tot, off);
+        }
+        if (lane == 0) {
+            s_pre = pre;
+            if (blockIdx.x == 0) {
+                *n_inst = (int64_t)tot;
+                count[Ttot] = (uint32_t)min(tot, cap);
+                if (tot > cap) set_status(status, CGS_ERR_CAPACITY);
+            }
+        }
+    }
+    if (blockIdx.x == 0 && threadIdx.x == 0) *nbig = 0u;   // the long-tile list starts empty
     __syncthreads();
-    if (order && threadIdx.x < kLenBuckets) {
-        uint32_t longer = 0;
-        for (int b = threadIdx.x + 1; b < kLenBuckets; b++) longer += btot[b];
-        offs[threadIdx.x] += longer;
-    }
-    const int64_t b0 = (int64_t)blockIdx.x * kScanSpan;
-    uint32_t c[kScanPer];
+    if (ONE && order) {
 #pragma unroll
-    for (int k = 0; k < kScanPer; k++) {
-        const int64_t t = b0 + k * kScanThreads + threadIdx.x;
-        c[k] = t < Ttot ? count[t] : 0u;
+        for (int k = 0; k < kScanPer; k++)
+            if (t0 + k < Ttot && lane == __ffs(peers[k]) - 1) atomicAdd(&btot[len_bucket(c[k])], __popc(peers[k]));
+        __syncthreads();
     }
-    unsigned long long run = s_pre;
-#pragma unroll
-    for (int k = 0; k < kScanPer; k++) {   // 1024 entries at a time, in tile order
-        unsigned long long incl = c[k];
+    // tiles in longer buckets: suffix sums within the warps of the first 256 threads, then
+    // across them
+    uint32_t longer = 0u;
+    if (order && threadIdx.x < 256u) {
+        const uint32_t own = threadIdx.x < kLenBuckets ? btot[threadIdx.x] : 0u;
+        uint32_t x = own;
 #pragma unroll
         for (int off = 1; off < 32; off <<= 1) {
-            const unsigned long long y = __shfl_up_sync(kFull, incl, off);
-            if (lane >= off) incl += y;
+            const uint32_t y = __shfl_down_sync(kFull, x, off);
+            if (lane + off < 32) x += y;
         }
-        if (lane == 31) wtot[w] = incl;
-        __syncthreads();
-        unsigned long long wpre = 0, btot_k = 0;
-        for (int i = 0; i < kScanThreads / 32; i++) {
-            const unsigned long long x = wtot[i];
-            wpre += i < w ? x : 0ull;
-            btot_k += x;
+        if (lane == 0) blong[w] = x;
+        longer = x - own;
+    }
+    unsigned long long wpre = lane < w ? wtot[lane] : 0ull;
+    static_assert(kScanThreads == 1024, "one warp total per lane");
+    for (int off = 16; off > 0; off >>= 1) wpre += __shfl_xor_sync(kFull, wpre, off);
+    unsigned long long st = (ONE ? 0ull : s_pre) + wpre + incl - tsum;
+    if (ONE && threadIdx.x == kScanThreads - 1) {
+        const unsigned long long tot = st + tsum;
+        *n_inst = (int64_t)tot;
+        count[Ttot] = (uint32_t)min(tot, cap);
+        if (tot > cap) set_status(status, CGS_ERR_CAPACITY);
+    }
+#pragma unroll
+    for (int k = 0; k < kScanPer; k++) {
+        const unsigned long long en = st + c[k];
+        if (t0 + k < Ttot) {
+            count[t0 + k] = (uint32_t)min(st, cap);
+            ranges[2 * (t0 + k)] = (uint32_t)min(st, cap);
+            ranges[2 * (t0 + k) + 1] = (uint32_t)min(en, cap);
         }
-        const int64_t t = b0 + k * kScanThreads + threadIdx.x;
-        if (t < Ttot) {
-            const unsigned long long st = run + wpre + incl - c[k], en = run + wpre + incl;
-            count[t] = (uint32_t)min(st, cap);
-            ranges[2 * t] = (uint32_t)min(st, cap);
-            ranges[2 * t + 1] = (uint32_t)min(en, cap);
-        }
-        run += btot_k;
-        __syncthreads();   // wtot is rewritten by the next round
+        st = en;
     }
     if (order) {
+        __syncthreads();   // blong
+        if (threadIdx.x < kLenBuckets) {
+            for (int i = w + 1; i < 8; i++) longer += blong[i];
+            offs[threadIdx.x] += longer;
+        }
+        __syncthreads();   // offs
 #pragma unroll
         for (int k = 0; k < kScanPer; k++) {
-            const int64_t t = b0 + k * kScanThreads + threadIdx.x;
-            if (t < Ttot) order[atomicAdd(&offs[len_bucket(c[k])], 1u)] = (uint32_t)t;
+            const int leader = __ffs(peers[k]) - 1;
+            uint32_t at = 0u;
+            if (t0 + k < Ttot && lane == leader) at = atomicAdd(&offs[len_bucket(c[k])], __popc(peers[k]));
+            at = __shfl_sync(kFull, at, leader);
+            if (t0 + k < Ttot) order[at + __popc(peers[k] & ((1u << lane) - 1u))] = (uint32_t)(t0 + k);
         }
     }
 }
@@ -1046,9 +1109,14 @@ cudaError_t bin_sort(const float *rec, int64_t n, int V, const Grid &g, void *ws
     else
         k_count<<<blocks, threads, 0, s>>>(r4, n, V, g, w.count);
     const int nsb = (int)((Ttot + kScanSpan - 1) / kScanSpan);
-    k_scan_part<<<nsb, kScanThreads, 0, s>>>(w.count, Ttot, w.part, w.bhist);
-    k_scan_out<<<nsb, kScanThreads, 0, s>>>(w.count, Ttot, capacity, w.part, w.bhist, nsb, ranges, order, n_inst,
-                                            w.nbig, status);
+    if (nsb == 1) {
+        k_scan_out<true><<<1, kScanThreads, 0, s>>>(w.count, Ttot, capacity, w.part, w.bhist, 1, ranges, order, n_inst,
+                                                    w.nbig, status);
+    } else {
+        k_scan_part<<<nsb, kScanThreads, 0, s>>>(w.count, Ttot, w.part, w.bhist);
+        k_scan_out<false><<<nsb, kScanThreads, 0, s>>>(w.count, Ttot, capacity, w.part, w.bhist, nsb, ranges, order,
+                                                       n_inst, w.nbig, status);
+    }
     if (agg)
         k_scatter_agg<<<agrid, kAggThreads, agg_smem, s>>>(r4, n, chunk, g, w.count, w.cursor, w.bcount, w.slotrec,
                                                              w.keys, capacity);
