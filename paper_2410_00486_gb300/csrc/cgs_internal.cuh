@@ -38,6 +38,24 @@ __device__ __forceinline__ void set_status(int32_t *st, int code)
     if (st) atomicCAS(st, 0, code);
 }
 
+// Sum of floats kept as an unevaluated pair (Knuth's two-sum), good to about 2^-45.
+struct PairSum {
+    float h = 0.f, l = 0.f;
+    __device__ __forceinline__ void add(float x)
+    {
+        const float s = __fadd_rn(h, x), b = __fsub_rn(s, h);
+        l = __fadd_rn(l, __fadd_rn(__fsub_rn(h, __fsub_rn(s, b)), __fsub_rn(x, b)));
+        h = s;
+    }
+    __device__ __forceinline__ void add(const PairSum &o)
+    {
+        add(o.h);
+        l = __fadd_rn(l, o.l);
+    }
+    // (an infinite or NaN h has made l a NaN)
+    __device__ __forceinline__ double value() const { return isfinite(h) ? (double)h + (double)l : (double)h; }
+};
+
 // Argument checks shared by every entry point that takes a cgs_config (host code).
 constexpr int kMaxViews = 1024;
 
