@@ -189,7 +189,7 @@ int cgs_raster_bwd(const float *rec, const uint32_t *vals, const uint32_t *range
     a.sgrad = slot_grad;
     a.work = work;
     const int bd = cfg->batch_depth_bwd ? cfg->batch_depth_bwd : cfg->batch_depth;
-    return cuda_status(raster_bwd(a, cfg->tile, bd, (cudaStream_t)stream));
+    return cuda_status(raster_bwd(a, cfg->tile, bd, num_sms(), (cudaStream_t)stream));
 }
 
 int cgs_preprocess_bwd(const float *params, int64_t n, const cgs_camera *cams, int32_t V, const cgs_config *cfg,

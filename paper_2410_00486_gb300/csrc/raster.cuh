@@ -65,7 +65,8 @@ __device__ __forceinline__ void item_tile(const uint32_t *order, const Grid &g, 
 // per-(warp, splat) reduction covers 32*PPT pixels.
 // The forward keeps two (its per-thread state is small and occupancy pays; four measured
 // slower), the backward eight: one warp per 16x16 tile, half the warp reductions per pixel
-// of four pixels, which were a third of its time (3.84 vs 4.04 ms on the 16-view window).
+// of four pixels, which were a third of its time (3.84 vs 4.04 ms on the 16-view window);
+// on windows of few tiles four or two, a part of the tile per warp.
 constexpr int kPPTFwd = 2;
 constexpr int kPPTBwd = 8;
 
@@ -82,10 +83,10 @@ __host__ __device__ constexpr int ppt_for()
 // rows), so a splat that covers few rows leaves whole p-steps of the warp idle; with
 // consecutive rows per thread every p-step would hold rows spread over the warp's span.
 template <int B, int P>
-__device__ __forceinline__ int thread_row0()
+__device__ __forceinline__ int thread_row0(int tid)
 {
     constexpr int G = B >= 32 ? 1 : 32 / B;
-    const int grp = (int)threadIdx.x / B;
+    const int grp = tid / B;
     return (grp / G) * G * P + grp % G;
 }
 template <int B>
@@ -165,6 +166,6 @@ __device__ __forceinline__ float staged_power(const float4 &t0, float hC, float 
 }
 
 cudaError_t raster_fwd(const RasterFwdArgs &a, int B, int BD, cudaStream_t s);
-cudaError_t raster_bwd(const RasterBwdArgs &a, int B, int BD, cudaStream_t s);
+cudaError_t raster_bwd(const RasterBwdArgs &a, int B, int BD, int sms, cudaStream_t s);
 
 }  // namespace cgs

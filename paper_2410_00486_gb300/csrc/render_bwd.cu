@@ -30,6 +30,10 @@
 // so 28 warps stay resident.  With a work counter the grid is persistent: as many blocks
 // as are resident on the GPU take (view, tile) items in the sort's longest-first order
 // from the counter until none is left.
+//
+// Windows of few tiles split each 16x16 tile into two or four parts (bwd_parts), a warp and
+// four or two pixels a thread each: one 160x120 view 44 -> 29 us, one 640x480 view of 40k
+// Gaussians 190 -> 127 us, three of 637x479 343 -> 280 us.
 #include "raster.cuh"
 
 namespace cgs {
@@ -48,39 +52,39 @@ constexpr int kRedRows = 33;   // 32 lanes and a zero row
 
 __device__ __forceinline__ float sgnf(float x) { return x > 0.f ? 1.f : (x < 0.f ? -1.f : 0.f); }
 
-template <int B, int BD>
-__global__ void __launch_bounds__(B *B / ppt_for<B, kPPTBwd>(), (min_blocks_for<B, kPPTBwd, kBwdMinWarps>())) k_render_bwd(RasterBwdArgs a)
+// Shared memory of one work item: the staged batch, the loss gradients of its pixels (pixel p
+// of thread t at [p NT + t]: three channels, depth) and a reduction buffer per warp.
+template <int BD, int PIX, int NW>
+struct BwdSmem {
+    float4 s0[BD], s1[BD], s2[BD];
+    uint32_t slot[BD];
+    uint32_t smax[NW];
+    __align__(16) float red[NW * kRedRows * kRedStride];
+    float4 gi[PIX];
+};
+
+// One work item: the tile at a place of the work order by NT threads of PPT pixels each, or
+// (S > 1) one of S parts of it by a warp on its own in a block of several: a half of eight
+// rows, or one of the four 8x8 blocks, whose short outline the fewest splats cross.
+template <int B, int BD, int NT, int PPT, int S, class Smem>
+__device__ __forceinline__ void bwd_item(const RasterBwdArgs &a, uint32_t place, int part, int tid, Smem &sm)
 {
-    constexpr int PPT = ppt_for<B, kPPTBwd>();
-    constexpr int NT = B * B / PPT;
     constexpr int NW = NT / 32;
-    __shared__ float4 s0[BD], s1[BD], s2[BD];
-    __shared__ uint32_t sslot[BD];
-    __shared__ uint32_t smax[NW];
-    __shared__ __align__(16) float red[NW * kRedRows * kRedStride];   // per warp
-    __shared__ float4 sgi[PPT * NT];   // per pixel p of thread t at [p NT + t]: dL/dimg (3 channels), dL/ddepth
-    __shared__ uint32_t s_item;
-    for (int i = threadIdx.x; i < NW * kRedStride; i += NT)   // the zero row of every warp's buffer
-        red[(i / kRedStride) * (kRedRows * kRedStride) + 32 * kRedStride + i % kRedStride] = 0.f;
-    const uint32_t n_items = (uint32_t)(a.g.Tv * a.V);
-    for (uint32_t it = 0;; it++) {
-    uint32_t item = blockIdx.x;
-    if (a.work) {
-        __syncthreads();   // the previous item's reads of s_item and of the shared state are done
-        if (threadIdx.x == 0) s_item = atomicAdd(a.work, 1u);
-        __syncthreads();
-        item = s_item;
-        if (item >= n_items) break;
-    } else if (it > 0) {
-        break;
-    }
+    constexpr bool kWarp = S > 1, kBlocks = S == 4;
+    float4 *s0 = sm.s0, *s1 = sm.s1, *s2 = sm.s2, *sgi = sm.gi;
+    uint32_t *sslot = sm.slot;
+    auto item_sync = [] {
+        if (kWarp) __syncwarp();
+        else __syncthreads();
+    };
+    const int lane = threadIdx.x & 31;
     int64_t tile;
     int view, tx, ty;
-    item_tile(a.order, a.g, tile, view, tx, ty, item);
-    const int lane = threadIdx.x & 31;
-    const int px = tx * B + (int)(threadIdx.x % B);
-    constexpr int G = row_step<B>();
-    const int py0 = ty * B + thread_row0<B, PPT>();   // row of pixel p: py0 + G p
+    item_tile(a.order, a.g, tile, view, tx, ty, place);
+    // row of pixel p: py0 + G p
+    constexpr int G = kBlocks ? 4 : row_step<B>();
+    const int px = tx * B + (kBlocks ? 8 * (part & 1) + (lane & 7) : tid % B);
+    const int py0 = ty * B + (kBlocks ? 8 * (part >> 1) + (lane >> 3) : part * (B / S) + thread_row0<B, PPT>(tid));
     const float fx = (float)px;
     const uint32_t start = a.ranges[2 * tile];
     const uint32_t len = a.ranges[2 * tile + 1] - start;
@@ -89,7 +93,7 @@ __global__ void __launch_bounds__(B *B / ppt_for<B, kPPTBwd>(), (min_blocks_for<
     // per-pixel state: transmittance, pixel gradients, and S = (colour behind) . gI +
     // (depth behind) gD, where "behind" starts as the background (no depth) and follows
     // R <- alpha c + (1 - alpha) R towards the front
-    float T[PPT], S[PPT];
+    float T[PPT], Sb[PPT];
     const float fy0 = (float)py0;   // row of pixel p: fy0 + G p (exact)
     uint32_t lst[PPT];
     uint32_t m = 0;
@@ -98,10 +102,10 @@ __global__ void __launch_bounds__(B *B / ppt_for<B, kPPTBwd>(), (min_blocks_for<
         const int py = py0 + G * p;
         lst[p] = 0;
         T[p] = 1.f;
-        S[p] = 0.f;
+        Sb[p] = 0.f;
         float gI0 = 0.f, gI1 = 0.f, gI2 = 0.f, gD = 0.f;
         if (!(px < a.g.W && py < a.g.H)) {
-            sgi[p * NT + threadIdx.x] = make_float4(0.f, 0.f, 0.f, 0.f);
+            sgi[p * NT + tid] = make_float4(0.f, 0.f, 0.f, 0.f);
             continue;
         }
         const size_t q = (size_t)py * a.g.W + px;
@@ -129,37 +133,66 @@ __global__ void __launch_bounds__(B *B / ppt_for<B, kPPTBwd>(), (min_blocks_for<
                 if (td > 0.f && cnt > 0) gD = w * a.lambda_d * sgnf(a.depth[pix] - td) / (float)cnt;
             }
         }
-        sgi[p * NT + threadIdx.x] = make_float4(gI0, gI1, gI2, gD);
-        S[p] = a.bg0 * gI0 + a.bg1 * gI1 + a.bg2 * gI2;
+        sgi[p * NT + tid] = make_float4(gI0, gI1, gI2, gD);
+        Sb[p] = a.bg0 * gI0 + a.bg1 * gI1 + a.bg2 * gI2;
         m = max(m, lst[p]);
     }
     // block-wide largest `last`: the walk starts there
     for (int off = 16; off > 0; off >>= 1) m = max(m, __shfl_xor_sync(kFull, m, off));
-    if (lane == 0) smax[threadIdx.x / 32] = m;
-    __syncthreads();
-    uint32_t maxlast = 0;
-    for (int i = 0; i < NW; i++) maxlast = max(maxlast, smax[i]);
+    uint32_t maxlast = kWarp ? m : 0u;
+    if (!kWarp) {
+        if (lane == 0) sm.smax[threadIdx.x / 32] = m;
+        __syncthreads();
+        for (int i = 0; i < NW; i++) maxlast = max(maxlast, sm.smax[i]);
+    }
 
-    for (int bend = (int)maxlast; bend > 0; bend -= BD) {
-        const int bstart = max(0, bend - BD);
-        const int nraw = bend - bstart;
-        __syncthreads();
-        // stage positions [bstart, bend) (every entry can reach the tile: the binning's test)
-        for (int c0 = 0; c0 < BD; c0 += NT) {
-            const int i = c0 + (int)threadIdx.x;
-            if (i >= nraw) break;
-            const uint32_t slot = __ldg(a.vals + start + bstart + i);
-            const float4 *r = a.rec + kRec4 * (size_t)slot;
-            const float4 r2 = __ldg(r + 2);
-            stage_splat(__ldg(r), __ldg(r + 1), r2.w, s0[i], s1[i]);
-            s2[i] = r2;
-            sslot[i] = slot;
+    // A part stages one splat a lane per batch, and the next batch's records are on their way
+    // while this one is walked (few warps: nothing else hides their latency)
+    constexpr bool kAhead = kWarp;
+    static_assert(!kAhead || BD == 32, "a splat a lane");
+    float4 n0, n1, n2;
+    uint32_t nslot = 0;
+    auto fetch = [&](int at) {   // the lane's splat of the batch ending at `at`
+        const int i = at - BD + lane;
+        if (i >= 0) {
+            nslot = __ldg(a.vals + start + i);
+            const float4 *r = a.rec + kRec4 * (size_t)nslot;
+            n0 = __ldg(r);
+            n1 = __ldg(r + 1);
+            n2 = __ldg(r + 2);
         }
-        __syncthreads();
+    };
+    if (kAhead) fetch((int)maxlast);
+    for (int bend = (int)maxlast; bend > 0; bend -= BD) {
+        const int bstart = kAhead ? bend - BD : max(0, bend - BD);   // below 0: the batch's first lanes are empty
+        const int nraw = bend - bstart;
+        item_sync();
+        // stage positions [bstart, bend) (every entry can reach the tile: the binning's test)
+        if (kAhead) {
+            if (bstart + lane >= 0) {
+                stage_splat(n0, n1, n2.w, s0[lane], s1[lane]);
+                s2[lane] = n2;
+                sslot[lane] = nslot;
+            }
+            fetch(bstart);
+        } else {
+            for (int c0 = 0; c0 < BD; c0 += NT) {
+                const int i = c0 + tid;
+                if (i >= nraw) break;
+                const uint32_t slot = __ldg(a.vals + start + bstart + i);
+                const float4 *r = a.rec + kRec4 * (size_t)slot;
+                const float4 r2 = __ldg(r + 2);
+                stage_splat(__ldg(r), __ldg(r + 1), r2.w, s0[i], s1[i]);
+                s2[i] = r2;
+                sslot[i] = slot;
+            }
+        }
+        item_sync();
+        const int j0 = kAhead ? max(0, -bstart) : 0;
         // two splats per loop trip, so one splat's loads and tests overlap the other's blend and
         // sums (3.470 -> 3.426 ms on the 16-view window; four per trip spill: 3.87 ms)
 #pragma unroll 2
-        for (int j = nraw - 1; j >= 0; j--) {
+        for (int j = nraw - 1; j >= j0; j--) {
             const uint32_t pos = (uint32_t)(bstart + j);   // list position of splat j
             const float4 q0 = s0[j];
             const float4 q1 = s1[j];
@@ -170,6 +203,7 @@ __global__ void __launch_bounds__(B *B / ppt_for<B, kPPTBwd>(), (min_blocks_for<
             // moments sum dp, sum dp dy, sum dp dy^2 of dp = dL/dpower (dx is shared)
             float gr = 0.f, gg = 0.f, gb = 0.f, gz = 0.f, go = 0.f, sdp = 0.f, sdpy = 0.f, sdpyy = 0.f;
             bool contrib = false;
+            unsigned who = 0u;   // lanes with a pixel that blends
             // pixels in pairs: a pair where either pixel blends runs both through the blend
             // (the other with G = 0, so alpha = 0 and its state is kept), so the two chains
             // interleave
@@ -189,12 +223,16 @@ __global__ void __launch_bounds__(B *B / ppt_for<B, kPPTBwd>(), (min_blocks_for<
                 // 3.297 ms on the 16-view window)
                 const bool pair = k[0] || k[1];
                 contrib = contrib || pair;
-                if (!__any_sync(kFull, pair)) continue;
+                if (PPT > 2 && !__any_sync(kFull, pair)) continue;
+                if (PPT == 2) {
+                    who = __ballot_sync(kFull, pair);
+                    if (who == 0u) break;
+                }
 #pragma unroll
                 for (int h = 0; h < 2; h++) {
                     const int p = p2 + h;
                     const float dy = dyv[h];
-                    const float4 gi = sgi[p * NT + threadIdx.x];   // dL/dimg, dL/ddepth of pixel p
+                    const float4 gi = sgi[p * NT + tid];   // dL/dimg, dL/ddepth of pixel p
                     const float G = k[h] ? exp2_fast(pw[h]) : 0.f;
                     const float araw = __fmul_rn(q1.y, G);
                     const float alpha = fminf(kAlphaMax, araw);
@@ -206,8 +244,8 @@ __global__ void __launch_bounds__(B *B / ppt_for<B, kPPTBwd>(), (min_blocks_for<
                     gb = fmaf(wT, gi.z, gb);
                     gz = fmaf(wT, gi.w, gz);
                     const float cg = fmaf(q1.z, gi.w, fmaf(q2.z, gi.z, fmaf(q2.y, gi.y, q2.x * gi.x)));
-                    const float diff = cg - S[p];
-                    S[p] = fmaf(alpha, diff, S[p]);
+                    const float diff = cg - Sb[p];
+                    Sb[p] = fmaf(alpha, diff, Sb[p]);
                     // dalpha/dpower = alpha, dalpha/dopacity = G, both 0 where alpha is clamped
                     const float dLda = araw > kAlphaMax ? 0.f : diff * T[p];
                     go = fmaf(dLda, G, go);
@@ -218,7 +256,7 @@ __global__ void __launch_bounds__(B *B / ppt_for<B, kPPTBwd>(), (min_blocks_for<
                     sdpyy = fmaf(dpy, dy, sdpyy);
                 }
             }
-            const unsigned who = __ballot_sync(kFull, contrib);
+            if (PPT > 2) who = __ballot_sync(kFull, contrib);
             if (who == 0u) continue;
             // raw moments of dp over this thread's pixels: sum dp dx, dp dy, dp dx^2, dp dx dy, dp dy^2
             const float m0 = sdp * dx, m3 = sdpy * dx;
@@ -245,7 +283,7 @@ __global__ void __launch_bounds__(B *B / ppt_for<B, kPPTBwd>(), (min_blocks_for<
                 // row, then lanes 10g + f (g < 3, f < 10) add field f over rows g, g + 3,
                 // g + 6, ... and three shuffles combine the groups (row stride 12 floats:
                 // the 16-byte stores are conflict-free, the column reads nearly so)
-                float *buf = red + (size_t)(threadIdx.x >> 5) * (kRedRows * kRedStride);
+                float *buf = sm.red + (kWarp ? 0 : (size_t)(threadIdx.x >> 5) * (kRedRows * kRedStride));
                 __syncwarp();   // the previous sum's column reads are done before the rows are rewritten
                 float4 *row = reinterpret_cast<float4 *>(buf + lane * kRedStride);
                 row[0] = make_float4(m0, sdpy, m0 * dx, m3);
@@ -280,53 +318,148 @@ __global__ void __launch_bounds__(B *B / ppt_for<B, kPPTBwd>(), (min_blocks_for<
             }
         }
     }
-    }   // work items
+}
+
+// The zero rows of a block's reduction buffers.
+template <int N>
+__device__ __forceinline__ void zero_rows(float (&red)[N], int t, int threads)
+{
+    for (int i = t; i < N / kRedRows; i += threads)
+        red[(i / kRedStride) * (kRedRows * kRedStride) + 32 * kRedStride + i % kRedStride] = 0.f;
+}
+
+// A block takes a tile at a time, the next one in the work order from the work counter (a
+// persistent launch), or its own.
+template <int B, int BD>
+__global__ void __launch_bounds__(B *B / ppt_for<B, kPPTBwd>(), (min_blocks_for<B, kPPTBwd, kBwdMinWarps>())) k_render_bwd(RasterBwdArgs a)
+{
+    constexpr int PPT = ppt_for<B, kPPTBwd>();
+    constexpr int NT = B * B / PPT;
+    __shared__ BwdSmem<BD, NT * PPT, NT / 32> sm;
+    __shared__ uint32_t s_item;
+    zero_rows(sm.red, threadIdx.x, NT);
+    const uint32_t n_items = (uint32_t)(a.g.Tv * a.V);
+    for (uint32_t it = 0;; it++) {
+        uint32_t item = blockIdx.x;
+        if (a.work) {
+            __syncthreads();   // the previous item's reads of s_item and of the shared state are done
+            if (threadIdx.x == 0) s_item = atomicAdd(a.work, 1u);
+            __syncthreads();
+            item = s_item;
+            if (item >= n_items) break;
+        } else if (it > 0) {
+            break;
+        }
+        bwd_item<B, BD, NT, PPT, 1>(a, item, 0, threadIdx.x, sm);
+    }
+}
+
+// Windows of few 16x16 tiles (bwd_parts): the warps of a block of four take parts of tiles,
+// each on its own.
+constexpr int kPartWarps = 4, kPartMinBlocks = 5;
+template <int S>
+__global__ void __launch_bounds__(32 * kPartWarps, kPartMinBlocks) k_render_bwd_parts(RasterBwdArgs a)
+{
+    __shared__ BwdSmem<32, 256 / S, 1> smem[kPartWarps];
+    auto &sm = smem[threadIdx.x >> 5];
+    const int lane = threadIdx.x & 31;
+    zero_rows(sm.red, lane, 32);
+    const uint32_t n_items = (uint32_t)(a.g.Tv * a.V) * S;
+    for (uint32_t it = 0;; it++) {
+        uint32_t item = blockIdx.x * kPartWarps + (threadIdx.x >> 5);
+        __syncwarp();   // the zero rows are written; the previous item's reads of the shared state are done
+        if (a.work) {
+            if (lane == 0) item = atomicAdd(a.work, 1u);
+            item = __shfl_sync(kFull, item, 0);
+        } else if (it > 0) {
+            break;
+        }
+        if (item >= n_items) break;
+        bwd_item<16, 32, 32, 8 / S, S>(a, item / S, (int)(item % S), lane, sm);
+    }
+}
+
+// Parts of a tile.  With one part the warp sums cover most pixels, which is best when the
+// window has work for the whole GPU; a window of few tiles is bound by the walk of its longest
+// list, one warp's chain of dependent steps, each shorter the fewer pixels the warp blends.
+// Measured (us, one, two and four parts): 80 tiles 52, 38, 29; 1200 tiles 193, 148, 127; 1900
+// tiles 242, 199, 166; 2394 tiles 142, 112, 110; 3225 tiles 321, 278, 335; 3600 tiles 386, 280,
+// 327; 5700 tiles 494, 524, 633; 9600 tiles 756, 838, 966.  Splitting only the longest lists'
+// tiles in four: 3225 tiles 314 to 395, 5700 tiles 493 to 602, never the best.
+static int bwd_parts(int64_t tiles, int sms)
+{
+    return tiles <= 16 * (int64_t)sms ? 4 : (tiles <= 32 * (int64_t)sms ? 2 : 1);
+}
+
+// Blocks of a persistent launch: as many as are resident on the GPU (queried once per device
+// and kernel), at most `items` of them; clears the work counter.
+template <class K>
+static cudaError_t persistent_blocks(const RasterBwdArgs &a, K kernel, int threads, int (&resident)[64], int sms,
+                                     int64_t &blocks, cudaStream_t s)
+{
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
+    if (!resident[dev]) {
+        int per_sm = 0;
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, threads, 0);
+        if (e != cudaSuccess) return e;
+        resident[dev] = max(1, per_sm) * max(1, sms);
+    }
+    blocks = min(blocks, (int64_t)resident[dev]);
+    return cudaMemsetAsync(a.work, 0, sizeof(uint32_t), s);
 }
 
 template <int B, int BD>
-static cudaError_t launch_bwd(const RasterBwdArgs &a, cudaStream_t s)
+static cudaError_t launch_bwd(const RasterBwdArgs &a, int sms, cudaStream_t s)
 {
     const int nt = B * B / ppt_for<B, kPPTBwd>();
     int64_t blocks = a.g.Tv * a.V;
     if (a.work) {
-        // persistent: the resident blocks of the whole GPU (queried once per device and shape)
         static int resident[64] = {0};
-        int dev = 0;
-        cudaError_t e = cudaGetDevice(&dev);
-        if (e != cudaSuccess) return e;
-        if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
-        if (!resident[dev]) {
-            int per_sm = 0, sms = 0;
-            e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_render_bwd<B, BD>, nt, 0);
-            if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-            if (e != cudaSuccess) return e;
-            resident[dev] = max(1, per_sm) * max(1, sms);
-        }
-        blocks = min(blocks, (int64_t)resident[dev]);
-        e = cudaMemsetAsync(a.work, 0, sizeof(uint32_t), s);
+        const cudaError_t e = persistent_blocks(a, k_render_bwd<B, BD>, nt, resident, sms, blocks, s);
         if (e != cudaSuccess) return e;
     }
     if (blocks > 0) k_render_bwd<B, BD><<<(unsigned)blocks, nt, 0, s>>>(a);
     return cudaGetLastError();
 }
 
-template <int B>
-static cudaError_t launch_bwd_bd(const RasterBwdArgs &a, int BD, cudaStream_t s)
+template <int S>
+static cudaError_t launch_bwd_parts(const RasterBwdArgs &a, int sms, cudaStream_t s)
 {
+    int64_t blocks = (a.g.Tv * a.V * S + kPartWarps - 1) / kPartWarps;
+    if (a.work) {
+        static int resident[64] = {0};
+        const cudaError_t e = persistent_blocks(a, k_render_bwd_parts<S>, 32 * kPartWarps, resident, sms, blocks, s);
+        if (e != cudaSuccess) return e;
+    }
+    k_render_bwd_parts<S><<<(unsigned)blocks, 32 * kPartWarps, 0, s>>>(a);
+    return cudaGetLastError();
+}
+
+template <int B>
+static cudaError_t launch_bwd_bd(const RasterBwdArgs &a, int BD, int sms, cudaStream_t s)
+{
+    if (B == 16) {
+        const int parts = bwd_parts(a.g.Tv * a.V, sms);
+        if (parts == 4) return launch_bwd_parts<4>(a, sms, s);
+        if (parts == 2) return launch_bwd_parts<2>(a, sms, s);
+    }
     switch (BD) {
-    case 32: return launch_bwd<B, 32>(a, s);
-    case 64: return launch_bwd<B, 64>(a, s);
-    case 128: return launch_bwd<B, 128>(a, s);
-    default: return launch_bwd<B, 256>(a, s);
+    case 32: return launch_bwd<B, 32>(a, sms, s);
+    case 64: return launch_bwd<B, 64>(a, sms, s);
+    case 128: return launch_bwd<B, 128>(a, sms, s);
+    default: return launch_bwd<B, 256>(a, sms, s);
     }
 }
 
-cudaError_t raster_bwd(const RasterBwdArgs &a, int B, int BD, cudaStream_t s)
+cudaError_t raster_bwd(const RasterBwdArgs &a, int B, int BD, int sms, cudaStream_t s)
 {
     switch (B) {
-    case 8: return launch_bwd_bd<8>(a, BD, s);
-    case 16: return launch_bwd_bd<16>(a, BD, s);
-    default: return launch_bwd_bd<32>(a, BD, s);
+    case 8: return launch_bwd_bd<8>(a, BD, sms, s);
+    case 16: return launch_bwd_bd<16>(a, BD, sms, s);
+    default: return launch_bwd_bd<32>(a, BD, sms, s);
     }
 }
 
