@@ -41,7 +41,7 @@ constexpr size_t kAggMaxSmem = 96 * 1024;   // per-view tile histogram in shared
 // 0.153 (49 blocks of 2048 slots for 152 SMs).
 // A small window takes smaller chunks, down to 256, until every SM has a block (one 640x480
 // view of 40k Gaussians: count 12.0 -> 9.9 us, 160x120 of 2k: 7.7 -> 4.8, scatter 6.3 -> 4.3;
-// one 1200x680 view of 100k, in chunks of 512: 25 and 29 us as before).
+// one 1200x680 view of 100k, in chunks of 512: 25 and 29 us as before, its large rects then).
 constexpr int kChunkLarge = 2048, kChunkSmall = 1024, kChunkMin = 256;
 static int chunk_for(int64_t n, int64_t V, int num_sms)
 {
@@ -201,14 +201,19 @@ __device__ __forceinline__ Rect reach_rect(const ReachPre &e, float u, float v, 
 // sum of their item counts, and hands out one item per lane and step; a lane finds the
 // slot owning item j by a 5-step binary search over the prefix (shuffles) and reads the
 // slot from the stage.  An item is one tile of the slot's reach rect (reach_rect,
-// row-major) to test, or, in the scatter pass for a slot with a recorded mask, one set
-// bit of the mask.
+// row-major) to test, or, in the scatter pass, one set bit of the slot's recorded mask.
+// Slots whose reach rect has more than kMaskTiles tiles are left for the end, when all warps
+// of the block test their tiles together: a splat near the camera covers hundreds of tiles,
+// and the warp that had it in its group kept the block waiting (one 1200x680 view of 100k
+// Gaussians: count 25 -> 15 us, scatter 30 -> 16 us; four of 90k: 42 -> 32 and 45 -> 26 us;
+// 16 of 300k: 220 -> 225 and 240 -> 229 us).
 // Slot bin records (SlotBin, 16 bytes per slot, written by the count pass for every slot
 // of the chunk): a slot whose reach rect has at most 64 tiles keeps one bit per tile
 // (row-major over that rect) saying whether it passed the reach test, with its depth bits
 // and the rect's first tile and width, so the scatter pass emits its tiles from the record
 // alone; a larger rect is marked for testing again; a slot that reaches no tile is zero.
 constexpr int kMaskTiles = 64;
+constexpr int kSegTiles = 128;   // tiles of a large rect a warp takes at a time
 // SlotBin = (mask low, mask high, depth bits, meta); meta is 0 (no tile), kBinLarge, or
 // kBinSmall | (width - 1) << 15 | first tile (tile id in the view, < 2^15).
 constexpr uint32_t kBinSmall = 0x80000000u, kBinLarge = 0x40000000u;
@@ -216,7 +221,7 @@ static_assert(kAggMaxSmem / sizeof(uint32_t) <= 32768, "first tile of a SlotBin 
 
 struct PairStage {      // one warp's 32 slots
     float4 a[32];       // u, v, 1/w (reach rect width w), depth bits
-    int4 b[32];         // reach rect's first tile (id in the view), w, mask kept, x0 | y0 << 16
+    int4 b[32];         // reach rect's first tile (id in the view), w, x0 | y0 << 16
     float4 c[32];       // reach test: A, 2B, C, t2
     float4 d[32];       //             ex, ey, B/C, B/A
     int4 e[32];         //             mode; tile mask low and high words
@@ -247,10 +252,45 @@ __device__ __forceinline__ int nth_bit64(uint64_t x, int k)
     return k < c ? nth_bit32(lo, k) : 32 + nth_bit32((uint32_t)(x >> 32), k - c);
 }
 
+// Slots of a chunk with large rects: position in the chunk << 16 | tiles of the rect.
+struct LargeList {
+    uint32_t n, slot[kChunkLarge];
+};
+static_assert(kChunkLarge <= 1 << 16 && kAggMaxSmem / sizeof(uint32_t) < 1 << 16, "a LargeList entry is one word");
+
+// Row and column of tile idx (row-major) of a rect of width w; inv = 1 / w rounded.
+__device__ __forceinline__ void rect_tile(int idx, int w, float inv, int &row, int &col)
+{
+    row = (int)(((float)idx + 0.5f) * inv);
+    col = idx - row * w;
+    if (col < 0) {           // the float quotient is within one of the exact one
+        row--;
+        col += w;
+    } else if (col >= w) {
+        row++;
+        col -= w;
+    }
+}
+
+// A visible slot's reach test and the tiles it may reach (none: T empty).
+__device__ __forceinline__ bool slot_reach(const float4 *__restrict__ rec, int64_t slot, const Grid &g, float &u,
+                                           float &v, uint32_t &zb, ReachPre &e, Rect &T)
+{
+    float z;
+    int r;
+    if (!load_slot(rec, slot, u, v, z, r)) return false;
+    const Rect R = tile_rect(u, v, r, g);
+    if (R.x1 <= R.x0 || R.y1 <= R.y0) return false;
+    e = load_reach(rec, slot, g);
+    T = reach_rect(e, u, v, R, g);
+    zb = __float_as_uint(z);
+    return true;
+}
+
 template <bool RECORD, class F>
 __device__ __forceinline__ void for_each_tile_pair(const float4 *__restrict__ rec, int64_t n, int view, int64_t s0,
-                                                   int64_t s1, const Grid &g, uint32_t *next, PairStage &st,
-                                                   uint4 *__restrict__ slotrec, F f)
+                                                   int64_t s1, const Grid &g, uint32_t *next, LargeList &large,
+                                                   PairStage &st, uint4 *__restrict__ slotrec, F f)
 {
     const int lane = threadIdx.x & 31;
     for (;;) {
@@ -261,13 +301,22 @@ __device__ __forceinline__ void for_each_tile_pair(const float4 *__restrict__ re
         if (wb >= s1) break;   // warp-uniform
         const int64_t gi = wb + lane;
         const int64_t slot = (int64_t)view * n + gi;
-        int cnt = 0, t0 = 0, w = 0, small = 0, xy0 = 0;
+        int cnt = 0, t0 = 0, w = 0, xy0 = 0;
         float u = 0.f, v = 0.f;
         uint32_t zb = 0u;
         ReachPre e{0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0};
         uint64_t mk = 0ull;
-        bool test = RECORD;   // slot's tiles come from the reach test (else from its mask)
-        if (!RECORD && gi < s1) {
+        bool big = false;
+        if (RECORD) {
+            Rect T;
+            if (gi < s1 && slot_reach(rec, slot, g, u, v, zb, e, T)) {
+                w = T.x1 - T.x0;
+                cnt = w * (T.y1 - T.y0);
+                t0 = T.y0 * g.Tx + T.x0;
+                xy0 = T.x0 | (T.y0 << 16);
+                big = cnt > kMaskTiles;
+            }
+        } else if (gi < s1) {
             const uint4 sb = slotrec[slot];
             if (sb.w & kBinSmall) {
                 mk = ((uint64_t)sb.y << 32) | sb.x;
@@ -275,30 +324,22 @@ __device__ __forceinline__ void for_each_tile_pair(const float4 *__restrict__ re
                 zb = sb.z;
                 w = (int)((sb.w >> 15) & 63u) + 1;
                 t0 = (int)(sb.w & 0x7fffu);
-                small = 1;
             } else if (sb.w & kBinLarge) {
-                test = true;
+                big = true;
+                cnt = (int)sb.x;
             }
         }
-        float z;
-        int r;
-        if (test && gi < s1 && load_slot(rec, slot, u, v, z, r)) {
-            const Rect R = tile_rect(u, v, r, g);
-            if (R.x1 > R.x0 && R.y1 > R.y0) {
-                e = load_reach(rec, slot, g);
-                const Rect T = reach_rect(e, u, v, R, g);
-                w = T.x1 - T.x0;
-                cnt = w * (T.y1 - T.y0);
-                t0 = T.y0 * g.Tx + T.x0;
-                xy0 = T.x0 | (T.y0 << 16);
-                small = RECORD && cnt <= kMaskTiles;
-                zb = __float_as_uint(z);
-            }
+        if (big) {
+            large.slot[atomicAdd(&large.n, 1u)] = (uint32_t)(gi - s0) << 16 | (uint32_t)cnt;
+            if (RECORD) slotrec[slot] = make_uint4((uint32_t)cnt, 0u, zb, kBinLarge);
+            cnt = 0;
         }
         st.a[lane] = make_float4(u, v, w ? 1.f / (float)w : 0.f, __uint_as_float(zb));
-        st.b[lane] = make_int4(t0, w, small, xy0);
-        st.c[lane] = make_float4(e.A, e.B2, e.C, e.t2);
-        st.d[lane] = make_float4(e.ex, e.ey, e.bc, e.ba);
+        st.b[lane] = make_int4(t0, w, xy0, 0);
+        if (RECORD) {
+            st.c[lane] = make_float4(e.A, e.B2, e.C, e.t2);
+            st.d[lane] = make_float4(e.ex, e.ey, e.bc, e.ba);
+        }
         st.e[lane] = make_int4(e.mode, (int)(uint32_t)mk, (int)(uint32_t)(mk >> 32), 0);
         __syncwarp();
         int incl = cnt;
@@ -317,28 +358,22 @@ __device__ __forceinline__ void for_each_tile_pair(const float4 *__restrict__ re
             const int oend = __shfl_sync(kFull, incl, L), ocnt = __shfl_sync(kFull, cnt, L);
             const int4 ob = st.b[L];
             const bool live = j < total;
-            const bool from_mask = !RECORD && ob.z;
             const int k = j - (oend - ocnt);
             bool pass = false;
             if (live) {
                 const float4 oa = st.a[L];
-                const int idx = from_mask ? nth_bit64(((uint64_t)(uint32_t)st.e[L].z << 32) | (uint32_t)st.e[L].y, k)
-                                          : k;   // row-major index into the reach rect
-                int row = (int)(((float)idx + 0.5f) * oa.z), col = idx - row * ob.y;
-                if (col < 0) {           // the float quotient is within one of the exact one
-                    row--;
-                    col += ob.y;
-                } else if (col >= ob.y) {
-                    row++;
-                    col -= ob.y;
-                }
+                // row-major index into the reach rect
+                const int idx = RECORD ? k
+                                       : nth_bit64(((uint64_t)(uint32_t)st.e[L].z << 32) | (uint32_t)st.e[L].y, k);
+                int row, col;
+                rect_tile(idx, ob.y, oa.z, row, col);
                 const int t = ob.x + row * g.Tx + col;
-                if (from_mask) {
-                    pass = true;
-                } else {
+                if (RECORD) {
                     const float4 oc = st.c[L], od = st.d[L];
                     const ReachPre oe{oc.x, oc.y, oc.z, oc.w, od.x, od.y, od.z, od.w, st.e[L].x};
-                    pass = in_tile(oe, oa.x, oa.y, (ob.w & 0xffff) + col, (ob.w >> 16) + row, g);
+                    pass = in_tile(oe, oa.x, oa.y, (ob.z & 0xffff) + col, (ob.z >> 16) + row, g);
+                } else {
+                    pass = true;
                 }
                 if (pass) {
                     const uint32_t oslot = (uint32_t)((int64_t)view * n + wb + L);
@@ -346,12 +381,11 @@ __device__ __forceinline__ void for_each_tile_pair(const float4 *__restrict__ re
                 }
             }
             if (RECORD) {
-                // this step's decisions for the masked slots: the first lane of each owner's
-                // run of lanes ORs the run's bits into the owner's mask (one writer per owner
-                // and step)
+                // this step's decisions: the first lane of each owner's run of lanes ORs the
+                // run's bits into the owner's mask (one writer per owner and step)
                 const unsigned bal = __ballot_sync(kFull, pass);
                 const int first = max(0, (oend - ocnt) - r0);
-                if (live && ob.z && lane == first) {
+                if (live && lane == first) {
                     const int runlen = min(oend - r0, 32) - first;
                     const uint32_t bits = (bal >> first) & (runlen >= 32 ? kFull : ((1u << runlen) - 1u));
                     const uint64_t m = (((uint64_t)(uint32_t)st.e[L].z << 32) | (uint32_t)st.e[L].y) |
@@ -362,16 +396,38 @@ __device__ __forceinline__ void for_each_tile_pair(const float4 *__restrict__ re
                 __syncwarp();
             }
         }
-        if (RECORD && gi < s1) {
-            uint4 sb = make_uint4(0u, 0u, 0u, 0u);
-            if (cnt > 0 && small)
-                sb = make_uint4((uint32_t)st.e[lane].y, (uint32_t)st.e[lane].z, zb,
-                                kBinSmall | ((uint32_t)(w - 1) << 15) | (uint32_t)t0);
-            else if (cnt > 0)
-                sb = make_uint4(0u, 0u, zb, kBinLarge);
-            slotrec[slot] = sb;
-        }
+        if (RECORD && gi < s1 && !big)
+            slotrec[slot] = cnt > 0 ? make_uint4((uint32_t)st.e[lane].y, (uint32_t)st.e[lane].z, zb,
+                                                 kBinSmall | ((uint32_t)(w - 1) << 15) | (uint32_t)t0)
+                                    : make_uint4(0u, 0u, 0u, 0u);
         __syncwarp();   // the stage is rewritten by the next group
+    }
+    // the large rects, in runs of kSegTiles tiles dealt to the warps in turn
+    __syncthreads();
+    const uint32_t nlarge = large.n;
+    const int warp = threadIdx.x >> 5, warps = blockDim.x >> 5;
+    int turn = warp;   // segments until this warp's next
+    for (uint32_t i = 0; i < nlarge; i++) {
+        const uint32_t en = large.slot[i];
+        const int cnt = (int)(en & 0xffffu), segs = (cnt + kSegTiles - 1) / kSegTiles;
+        if (turn < segs) {   // warp-uniform
+            const int64_t slot = (int64_t)view * n + s0 + (en >> 16);
+            float u, v;
+            uint32_t zb;
+            ReachPre e;
+            Rect T;
+            slot_reach(rec, slot, g, u, v, zb, e, T);
+            const int w = T.x1 - T.x0;
+            const float inv = 1.f / (float)w;
+            const uint64_t key = ((uint64_t)zb << 32) | (uint64_t)(uint32_t)slot;
+            for (; turn < segs; turn += warps)
+                for (int idx = turn * kSegTiles + lane; idx < min(cnt, (turn + 1) * kSegTiles); idx += 32) {
+                    int row, col;
+                    rect_tile(idx, w, inv, row, col);
+                    if (in_tile(e, u, v, T.x0 + col, T.y0 + row, g)) f((T.y0 + row) * g.Tx + T.x0 + col, key);
+                }
+        }
+        turn -= segs;
     }
 }
 
@@ -391,10 +447,11 @@ k_count_agg(const float4 *__restrict__ rec, int64_t n, int chunk, Grid g, uint32
     const int64_t s0 = (int64_t)blockIdx.x * chunk;
     const int64_t s1 = min(n, s0 + chunk);
     __shared__ uint32_t next;
+    __shared__ LargeList large;
     for (int t = threadIdx.x; t < g.Tv; t += blockDim.x) hist[t] = 0;
-    if (threadIdx.x == 0) next = 0;
+    if (threadIdx.x == 0) next = large.n = 0;
     __syncthreads();
-    for_each_tile_pair<true>(rec, n, view, s0, s1, g, &next, stage[threadIdx.x >> 5], slotrec,
+    for_each_tile_pair<true>(rec, n, view, s0, s1, g, &next, large, stage[threadIdx.x >> 5], slotrec,
                              [&](int t, uint64_t) { atomicAdd(&hist[t], 1u); });
     __syncthreads();
     uint32_t *base = count + (int64_t)view * g.Tv;
@@ -624,7 +681,8 @@ k_scatter_agg(const float4 *__restrict__ rec, int64_t n, int chunk, Grid g, cons
     const int64_t tbase = (int64_t)view * g.Tv;
     const uint32_t *mine = bcount + ((int64_t)view * gridDim.x + blockIdx.x) * g.Tv;
     __shared__ uint32_t next;
-    if (threadIdx.x == 0) next = 0;
+    __shared__ LargeList large;
+    if (threadIdx.x == 0) next = large.n = 0;
     for (int t0 = threadIdx.x; t0 < g.Tv; t0 += 4 * blockDim.x) {   // four tiles in flight
         uint32_t c[4], st4[4], r[4];
 #pragma unroll
@@ -645,7 +703,7 @@ k_scatter_agg(const float4 *__restrict__ rec, int64_t n, int chunk, Grid g, cons
         }
     }
     __syncthreads();
-    for_each_tile_pair<false>(rec, n, view, s0, s1, g, &next, stage[threadIdx.x >> 5], slotrec,
+    for_each_tile_pair<false>(rec, n, view, s0, s1, g, &next, large, stage[threadIdx.x >> 5], slotrec,
                               [&](int t, uint64_t key) {
                                   const uint64_t pos = atomicAdd(&hist[t], 1u);
                                   if (pos < (uint64_t)capacity) keys[pos] = key;
@@ -1123,12 +1181,16 @@ cudaError_t bin_sort(const float *rec, int64_t n, int V, const Grid &g, void *ws
     else
         k_scatter<<<blocks, threads, 0, s>>>(r4, n, V, g, w.count, w.cursor, w.keys, capacity);
     k_sort_tiles<<<(unsigned)Ttot, kSortThreadsS, 0, s>>>(ranges, w.keys, vals, w.mid, w.nmid);
-    k_sort_tiles_l<<<(unsigned)std::min<int64_t>(Ttot, (int64_t)num_sms * 4), kSortThreadsL, 0, s>>>(
-        ranges, w.keys, vals, w.mid, w.nmid, w.big, w.nbig);
-    const size_t big_smem = sizeof(uint64_t) * kBigCap;
-    e = cudaFuncSetAttribute(k_sort_big, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)big_smem);
-    if (e != cudaSuccess) return e;
-    k_sort_big<<<num_sms, kBigThreads, big_smem, s>>>(ranges, w.keys, vals, w.big, w.nbig);
+    // a list holds a slot at most once, so no more than n of them (an empty launch is 3 us)
+    if (n > kSortCapS)
+        k_sort_tiles_l<<<(unsigned)std::min<int64_t>(Ttot, (int64_t)num_sms * 4), kSortThreadsL, 0, s>>>(
+            ranges, w.keys, vals, w.mid, w.nmid, w.big, w.nbig);
+    if (n > kSmallCap) {
+        const size_t big_smem = sizeof(uint64_t) * kBigCap;
+        e = cudaFuncSetAttribute(k_sort_big, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)big_smem);
+        if (e != cudaSuccess) return e;
+        k_sort_big<<<num_sms, kBigThreads, big_smem, s>>>(ranges, w.keys, vals, w.big, w.nbig);
+    }
     return cudaGetLastError();
 }
 
