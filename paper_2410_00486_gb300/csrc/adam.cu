@@ -62,6 +62,7 @@ __device__ __forceinline__ void bias_corrections(AdamArgs &a)
 // The step held on the device, and the regulariser's sum started at zero, before the update.
 __global__ void k_step_inc(int32_t *step, float *loss_o)
 {
+    pdl_begin(step, loss_o);
     *step += 1;
     if (loss_o) *loss_o = 0.f;
 }
@@ -83,6 +84,7 @@ __device__ __forceinline__ float adam_elem(int64_t i, float p, float g, float &m
 
 __global__ void __launch_bounds__(256) k_adam_vec(AdamArgs a)
 {
+    pdl_begin(a.g);
     float osum = 0.f;
     const int64_t n4 = a.total / 4;
     float4 *p4 = reinterpret_cast<float4 *>(a.p);
@@ -130,6 +132,7 @@ __global__ void __launch_bounds__(256) k_adam_vec(AdamArgs a)
 
 __global__ void __launch_bounds__(256) k_adam_scalar(AdamArgs a)
 {
+    pdl_begin(a.g);
     bias_corrections(a);
     float osum = 0.f;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < a.total; i += (int64_t)gridDim.x * blockDim.x) {
@@ -173,7 +176,7 @@ cudaError_t adam(float *p, const float *g, float *m, float *v, int64_t n, int de
     a.loss_o = loss_o;
     a.step_dev = step_dev;
     if (step_dev) {
-        k_step_inc<<<1, 1, 0, s>>>(step_dev, loss_o);
+        launch(k_step_inc, 1, 1, 0, s, step_dev, loss_o);
         cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) return e;
     } else if (loss_o) {
@@ -185,9 +188,9 @@ cudaError_t adam(float *p, const float *g, float *m, float *v, int64_t n, int de
     const int64_t work = aligned ? (L.total + 3) / 4 : L.total;
     const int blocks = (int)std::min<int64_t>((work + threads - 1) / threads, (int64_t)num_sms * 8);
     if (aligned)
-        k_adam_vec<<<blocks, threads, 0, s>>>(a);
+        launch(k_adam_vec, blocks, threads, 0, s, a);
     else
-        k_adam_scalar<<<blocks, threads, 0, s>>>(a);
+        launch(k_adam_scalar, blocks, threads, 0, s, a);
     return cudaGetLastError();
 }
 
@@ -195,6 +198,7 @@ __global__ void __launch_bounds__(256)
 k_densify(const float4 *__restrict__ rec, const float4 *__restrict__ sgrad, int64_t n, int V, float halfW, float halfH,
           float *__restrict__ accum, float *__restrict__ denom, float *__restrict__ maxr)
 {
+    pdl_begin(rec, sgrad, accum, denom, maxr);
     const int64_t total = (int64_t)V * n;
     for (int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; s < total; s += (int64_t)gridDim.x * blockDim.x) {
         const int r = __float_as_int(__ldg(reinterpret_cast<const float *>(rec + kRec4 * s) + 7));
@@ -213,8 +217,8 @@ cudaError_t densify_stats(const float *rec, const float *sgrad, int64_t n, int V
 {
     const int64_t total = (int64_t)V * n;
     const int blocks = (int)std::min<int64_t>((total + 255) / 256, (int64_t)num_sms * 16);
-    k_densify<<<blocks, 256, 0, s>>>(reinterpret_cast<const float4 *>(rec), reinterpret_cast<const float4 *>(sgrad), n,
-                                     V, 0.5f * (float)g.W, 0.5f * (float)g.H, accum, denom, maxr);
+    launch(k_densify, blocks, 256, 0, s, reinterpret_cast<const float4 *>(rec),
+           reinterpret_cast<const float4 *>(sgrad), n, V, 0.5f * (float)g.W, 0.5f * (float)g.H, accum, denom, maxr);
     return cudaGetLastError();
 }
 

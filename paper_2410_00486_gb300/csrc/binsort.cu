@@ -151,6 +151,7 @@ __device__ __forceinline__ bool in_tile(const ReachPre &e, float u, float v, int
 
 __global__ void k_count(const float4 *__restrict__ rec, int64_t n, int V, Grid g, uint32_t *__restrict__ count)
 {
+    pdl_begin(rec, count);
     const int64_t total = (int64_t)V * n;
     for (int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; s < total; s += (int64_t)gridDim.x * blockDim.x) {
         float u, v, z;
@@ -440,6 +441,7 @@ __global__ void __launch_bounds__(kAggThreads, kAggMinBlocks)
 k_count_agg(const float4 *__restrict__ rec, int64_t n, int chunk, Grid g, uint32_t *__restrict__ count,
             uint32_t *__restrict__ bcount, uint4 *__restrict__ slotrec)
 {
+    pdl_begin(rec, count, bcount, slotrec);
     extern __shared__ float4 smem_agg[];
     PairStage *stage = reinterpret_cast<PairStage *>(smem_agg);
     uint32_t *hist = reinterpret_cast<uint32_t *>(reinterpret_cast<char *>(smem_agg) + kStageBytes);
@@ -478,6 +480,7 @@ __global__ void __launch_bounds__(kScanThreads)
 k_scan_part(const uint32_t *__restrict__ count, int64_t Ttot, unsigned long long *__restrict__ part,
             uint32_t *__restrict__ bhist)
 {
+    pdl_begin(count, part, bhist);
     __shared__ unsigned long long wsum[kScanThreads / 32];
     __shared__ uint32_t hist[kLenBuckets];
     if (threadIdx.x < kLenBuckets) hist[threadIdx.x] = 0u;
@@ -521,6 +524,7 @@ k_scan_out(uint32_t *__restrict__ count, int64_t Ttot, int64_t capacity, const u
            uint32_t *__restrict__ order, int64_t *__restrict__ n_inst, uint32_t *__restrict__ nbig,
            int32_t *__restrict__ status)
 {
+    pdl_begin(count, part, bhist, ranges, order, n_inst, nbig, status);
     __shared__ unsigned long long wtot[kScanThreads / 32];
     __shared__ unsigned long long s_pre;
     __shared__ uint32_t btot[kLenBuckets], offs[kLenBuckets], blong[8];
@@ -644,6 +648,7 @@ __global__ void k_scatter(const float4 *__restrict__ rec, int64_t n, int V, Grid
                           const uint32_t *__restrict__ start, uint32_t *__restrict__ cursor,
                           uint64_t *__restrict__ keys, int64_t capacity)
 {
+    pdl_begin(rec, start, cursor, keys);
     const int64_t total = (int64_t)V * n;
     for (int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; s < total; s += (int64_t)gridDim.x * blockDim.x) {
         float u, v, z;
@@ -671,6 +676,7 @@ k_scatter_agg(const float4 *__restrict__ rec, int64_t n, int chunk, Grid g, cons
               uint32_t *__restrict__ cursor, const uint32_t *__restrict__ bcount, uint4 *__restrict__ slotrec,
               uint64_t *__restrict__ keys, int64_t capacity)
 {
+    pdl_begin(rec, start, cursor, bcount, slotrec, keys);
     extern __shared__ float4 smem_agg[];
     PairStage *stage = reinterpret_cast<PairStage *>(smem_agg);
     uint32_t *hist = reinterpret_cast<uint32_t *>(reinterpret_cast<char *>(smem_agg) + kStageBytes);  // run positions
@@ -1059,6 +1065,7 @@ __global__ void __launch_bounds__(kSortThreadsS)
 k_sort_tiles(const uint32_t *__restrict__ ranges, const uint64_t *__restrict__ keys, uint32_t *__restrict__ vals,
              uint32_t *__restrict__ mid, uint32_t *__restrict__ nmid)
 {
+    pdl_begin(ranges, keys, vals, mid, nmid);
     __shared__ SortSmem<kSortThreadsS, kSortCapS> sm;
     const int64_t t = blockIdx.x;
     const uint32_t st = ranges[2 * t], en = ranges[2 * t + 1];
@@ -1081,6 +1088,7 @@ k_sort_tiles_l(const uint32_t *__restrict__ ranges, const uint64_t *__restrict__
                const uint32_t *__restrict__ mid, const uint32_t *__restrict__ nmid, uint32_t *__restrict__ big,
                uint32_t *__restrict__ nbig)
 {
+    pdl_begin(ranges, keys, vals, mid, nmid, big, nbig);
     __shared__ SortSmem<kSortThreadsL, kSmallCap> sm;
     const uint32_t nm = *nmid;
     for (uint32_t mi = blockIdx.x; mi < nm; mi += gridDim.x) {   // block-uniform
@@ -1099,6 +1107,7 @@ __global__ void __launch_bounds__(kBigThreads)
 k_sort_big(const uint32_t *__restrict__ ranges, uint64_t *__restrict__ keys, uint32_t *__restrict__ vals,
            const uint32_t *__restrict__ big, const uint32_t *__restrict__ nbig)
 {
+    pdl_begin(ranges, keys, vals, big, nbig);
     extern __shared__ uint64_t sbig[];
     const uint32_t nb = *nbig;
     for (uint32_t bi = blockIdx.x; bi < nb; bi += gridDim.x) {
@@ -1163,33 +1172,33 @@ cudaError_t bin_sort(const float *rec, int64_t n, int V, const Grid &g, void *ws
     const int threads = 256;
     const int blocks = (int)std::min<int64_t>((slots + threads - 1) / threads, (int64_t)num_sms * 16);
     if (agg)
-        k_count_agg<<<agrid, kAggThreads, agg_smem, s>>>(r4, n, chunk, g, w.count, w.bcount, w.slotrec);
+        launch(k_count_agg, agrid, kAggThreads, agg_smem, s, r4, n, chunk, g, w.count, w.bcount, w.slotrec);
     else
-        k_count<<<blocks, threads, 0, s>>>(r4, n, V, g, w.count);
+        launch(k_count, blocks, threads, 0, s, r4, n, V, g, w.count);
     const int nsb = (int)((Ttot + kScanSpan - 1) / kScanSpan);
     if (nsb == 1) {
-        k_scan_out<true><<<1, kScanThreads, 0, s>>>(w.count, Ttot, capacity, w.part, w.bhist, 1, ranges, order, n_inst,
-                                                    w.nbig, status);
+        launch(k_scan_out<true>, 1, kScanThreads, 0, s, w.count, Ttot, capacity, w.part, w.bhist, 1, ranges, order,
+               n_inst, w.nbig, status);
     } else {
-        k_scan_part<<<nsb, kScanThreads, 0, s>>>(w.count, Ttot, w.part, w.bhist);
-        k_scan_out<false><<<nsb, kScanThreads, 0, s>>>(w.count, Ttot, capacity, w.part, w.bhist, nsb, ranges, order,
-                                                       n_inst, w.nbig, status);
+        launch(k_scan_part, nsb, kScanThreads, 0, s, w.count, Ttot, w.part, w.bhist);
+        launch(k_scan_out<false>, nsb, kScanThreads, 0, s, w.count, Ttot, capacity, w.part, w.bhist, nsb, ranges, order,
+               n_inst, w.nbig, status);
     }
     if (agg)
-        k_scatter_agg<<<agrid, kAggThreads, agg_smem, s>>>(r4, n, chunk, g, w.count, w.cursor, w.bcount, w.slotrec,
-                                                             w.keys, capacity);
+        launch(k_scatter_agg, agrid, kAggThreads, agg_smem, s, r4, n, chunk, g, w.count, w.cursor, w.bcount, w.slotrec,
+               w.keys, capacity);
     else
-        k_scatter<<<blocks, threads, 0, s>>>(r4, n, V, g, w.count, w.cursor, w.keys, capacity);
-    k_sort_tiles<<<(unsigned)Ttot, kSortThreadsS, 0, s>>>(ranges, w.keys, vals, w.mid, w.nmid);
+        launch(k_scatter, blocks, threads, 0, s, r4, n, V, g, w.count, w.cursor, w.keys, capacity);
+    launch(k_sort_tiles, (unsigned)Ttot, kSortThreadsS, 0, s, ranges, w.keys, vals, w.mid, w.nmid);
     // a list holds a slot at most once, so no more than n of them (an empty launch is 3 us)
     if (n > kSortCapS)
-        k_sort_tiles_l<<<(unsigned)std::min<int64_t>(Ttot, (int64_t)num_sms * 4), kSortThreadsL, 0, s>>>(
-            ranges, w.keys, vals, w.mid, w.nmid, w.big, w.nbig);
+        launch(k_sort_tiles_l, (unsigned)std::min<int64_t>(Ttot, (int64_t)num_sms * 4), kSortThreadsL, 0, s, ranges,
+               w.keys, vals, w.mid, w.nmid, w.big, w.nbig);
     if (n > kSmallCap) {
         const size_t big_smem = sizeof(uint64_t) * kBigCap;
         e = cudaFuncSetAttribute(k_sort_big, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)big_smem);
         if (e != cudaSuccess) return e;
-        k_sort_big<<<num_sms, kBigThreads, big_smem, s>>>(ranges, w.keys, vals, w.big, w.nbig);
+        launch(k_sort_big, num_sms, kBigThreads, big_smem, s, ranges, w.keys, vals, w.big, w.nbig);
     }
     return cudaGetLastError();
 }

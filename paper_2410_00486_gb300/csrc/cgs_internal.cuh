@@ -5,6 +5,8 @@
 #include <math.h>
 #include <stdint.h>
 
+#include <utility>
+
 #include "cgs.h"
 
 namespace cgs {
@@ -30,6 +32,46 @@ __host__ __device__ inline Layout param_layout(int64_t n, int deg)
     L.rest = 14 * n;
     L.total = 14 * n + 3 * (int64_t)(L.K - 1) * n;
     return L;
+}
+
+// Programmatic dependent launch.  A kernel launched with launch() may be placed on the GPU
+// while its predecessor in the stream still drains, which hides its launch latency.  Every
+// such kernel begins with pdl_begin(): it lets its own successor be placed in turn, then waits
+// until everything before it in the stream is complete and visible (the predecessor itself
+// came back from this wait, so completion is transitive).  The kernel's pointers go through
+// pdl_begin() so that no read, not even one the compiler takes for a read of constant memory,
+// can be moved ahead of the wait.  Behind anything but such a kernel the launch is an
+// ordinary one.  The chain of an iteration uses it: four views' render 462 -> 440 us, three
+// views with the SSIM loss 501 -> 478, one 640x480 view 212 -> 208, Adam's two kernels 105 ->
+// 100.  The loss of Eq. 9 and density control gained nothing from it (197 -> 222 and 119 -> 127
+// us, their loads no longer read-only ones) and are launched the ordinary way.
+template <class T>
+__device__ __forceinline__ void after_wait(T &pointer)
+{
+    asm volatile("" : "+l"(pointer));
+}
+template <class... T>
+__device__ __forceinline__ void pdl_begin(T &...pointers)
+{
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    (after_wait(pointers), ...);
+}
+
+template <class... K, class... A>
+inline cudaError_t launch(void (*kernel)(K...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, A &&...args)
+{
+    cudaLaunchAttribute attr = {};
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, std::forward<A>(args)...);
 }
 
 // Record a device-side condition; the first one wins.

@@ -333,6 +333,7 @@ __global__ void __launch_bounds__(kPreThreads)
 k_preprocess(const float *__restrict__ P, int64_t n, const cgs_camera *__restrict__ cams, int V,
              Grid grid, float near_z, float4 *__restrict__ rec, float4 *__restrict__ sgrad)
 {
+    pdl_begin(P, cams, rec, sgrad);
     extern __shared__ __align__(16) float sm[];
     const int64_t g0 = (int64_t)blockIdx.x * kGB;
     const int cnt = (int)min((int64_t)kGB, n - g0);
@@ -530,6 +531,7 @@ k_preprocess_bwd(const float *__restrict__ P, int64_t n, const cgs_camera *__res
                  float *__restrict__ pgrad, int accumulate, float *__restrict__ accum,
                  float *__restrict__ denom, float *__restrict__ max_r2d)
 {
+    pdl_begin(P, cams, rec, sgrad, pgrad, accum, denom, max_r2d);
     constexpr int K = (DEG + 1) * (DEG + 1);
     constexpr int R3 = 3 * (K - 1);
     extern __shared__ __align__(16) float sm[];
@@ -661,7 +663,7 @@ static cudaError_t launch_pre(const float *P, int64_t n, const cgs_camera *cams,
     if (e != cudaSuccess) return e;
     int blocks = (int)((n + kGB - 1) / kGB);
     // one view has an item for half of the threads only
-    k<<<blocks, V == 1 ? kGB : kPreThreads, smem, s>>>(P, n, cams, V, g, near_z, rec, sgrad);
+    launch(k, blocks, V == 1 ? kGB : kPreThreads, smem, s, P, n, cams, V, g, near_z, rec, sgrad);
     return cudaGetLastError();
 }
 
@@ -675,8 +677,8 @@ static cudaError_t launch_pre_bwd(const float *P, int64_t n, const cgs_camera *c
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     int blocks = (int)((n + kGB - 1) / kGB);
-    k<<<blocks, kPreThreads, smem, s>>>(P, n, cams, V, g, near_z, rec, sgrad, pgrad, accumulate, accum,
-                                        denom, maxr);
+    launch(k, blocks, kPreThreads, smem, s, P, n, cams, V, g, near_z, rec, sgrad, pgrad, accumulate, accum,
+           denom, maxr);
     return cudaGetLastError();
 }
 

@@ -333,6 +333,7 @@ __device__ __forceinline__ void zero_rows(float (&red)[N], int t, int threads)
 template <int B, int BD>
 __global__ void __launch_bounds__(B *B / ppt_for<B, kPPTBwd>(), (min_blocks_for<B, kPPTBwd, kBwdMinWarps>())) k_render_bwd(RasterBwdArgs a)
 {
+    pdl_begin();   // the read-only loads below are addressed by what is read after the wait
     constexpr int PPT = ppt_for<B, kPPTBwd>();
     constexpr int NT = B * B / PPT;
     __shared__ BwdSmem<BD, NT * PPT, NT / 32> sm;
@@ -360,6 +361,7 @@ constexpr int kPartWarps = 4, kPartMinBlocks = 5;
 template <int S>
 __global__ void __launch_bounds__(32 * kPartWarps, kPartMinBlocks) k_render_bwd_parts(RasterBwdArgs a)
 {
+    pdl_begin();   // the read-only loads below are addressed by what is read after the wait
     __shared__ BwdSmem<32, 256 / S, 1> smem[kPartWarps];
     auto &sm = smem[threadIdx.x >> 5];
     const int lane = threadIdx.x & 31;
@@ -421,7 +423,7 @@ static cudaError_t launch_bwd(const RasterBwdArgs &a, int sms, cudaStream_t s)
         const cudaError_t e = persistent_blocks(a, k_render_bwd<B, BD>, nt, resident, sms, blocks, s);
         if (e != cudaSuccess) return e;
     }
-    if (blocks > 0) k_render_bwd<B, BD><<<(unsigned)blocks, nt, 0, s>>>(a);
+    if (blocks > 0) launch(k_render_bwd<B, BD>, (unsigned)blocks, nt, 0, s, a);
     return cudaGetLastError();
 }
 
@@ -434,7 +436,7 @@ static cudaError_t launch_bwd_parts(const RasterBwdArgs &a, int sms, cudaStream_
         const cudaError_t e = persistent_blocks(a, k_render_bwd_parts<S>, 32 * kPartWarps, resident, sms, blocks, s);
         if (e != cudaSuccess) return e;
     }
-    k_render_bwd_parts<S><<<(unsigned)blocks, 32 * kPartWarps, 0, s>>>(a);
+    launch(k_render_bwd_parts<S>, (unsigned)blocks, 32 * kPartWarps, 0, s, a);
     return cudaGetLastError();
 }
 

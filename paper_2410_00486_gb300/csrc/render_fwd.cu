@@ -18,6 +18,7 @@ __device__ constexpr float kNoRow = __builtin_nanf("");
 template <int B, int BD, bool CKPT, bool COUNT>
 __global__ void __launch_bounds__(B *B / ppt_for<B, kPPTFwd>(), (min_blocks_for<B, kPPTFwd, kFwdMinWarps>())) k_render_fwd(RasterFwdArgs a)
 {
+    pdl_begin();   // the read-only loads below are addressed by what is read after the wait
     constexpr int PPT = ppt_for<B, kPPTFwd>();
     constexpr int NT = B * B / PPT;
     constexpr int NW = NT / 32;
@@ -193,6 +194,7 @@ k_loss_reduce(const float *__restrict__ partials, int64_t Tv, const float *__res
               float lambda_d, float *__restrict__ loss_view, int32_t *__restrict__ depth_count,
               int32_t *__restrict__ status)
 {
+    pdl_begin(partials, weight, loss_view, depth_count, status);
     constexpr int NW = kLossThreads / 32;
     __shared__ PairSum sh[3][NW];
     const int v = blockIdx.x, lane = threadIdx.x & 31, w = threadIdx.x >> 5;
@@ -236,11 +238,11 @@ static cudaError_t launch_fwd(const RasterFwdArgs &a, cudaStream_t s)
     const int64_t items = a.g.Tv * a.V;
     const int nt = B * B / ppt_for<B, kPPTFwd>();
     if (a.ck4)   // the checkpointing forward does not count blended pairs
-        k_render_fwd<B, BD, true, false><<<(unsigned)items, nt, 0, s>>>(a);
+        launch(k_render_fwd<B, BD, true, false>, (unsigned)items, nt, 0, s, a);
     else if (a.count_blend)
-        k_render_fwd<B, BD, false, true><<<(unsigned)items, nt, 0, s>>>(a);
+        launch(k_render_fwd<B, BD, false, true>, (unsigned)items, nt, 0, s, a);
     else
-        k_render_fwd<B, BD, false, false><<<(unsigned)items, nt, 0, s>>>(a);
+        launch(k_render_fwd<B, BD, false, false>, (unsigned)items, nt, 0, s, a);
     return cudaGetLastError();
 }
 
@@ -268,7 +270,8 @@ cudaError_t loss_reduce(const float *partials, const Grid &g, int V, const float
                         float *loss_view, int32_t *depth_count, int32_t *status, cudaStream_t s)
 {
     const double inv3HW = 1.0 / (3.0 * (double)g.W * (double)g.H);
-    k_loss_reduce<<<V, kLossThreads, 0, s>>>(partials, g.Tv, weight, inv3HW, lambda_d, loss_view, depth_count, status);
+    launch(k_loss_reduce, V, kLossThreads, 0, s, partials, g.Tv, weight, inv3HW, lambda_d, loss_view, depth_count,
+           status);
     return cudaGetLastError();
 }
 

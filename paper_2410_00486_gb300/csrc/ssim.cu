@@ -435,8 +435,8 @@ int cgs_ssim_loss(const float *img, const float *tgt_rgb, const float *depth, co
     if (e == cudaSuccess) {
         k_ssim_fwd<<<grid, kSsimThreads, 0, s>>>(img, tgt_rgb, W, H, steps, t, amap, bmap, cmap, acc);
         k_ssim_bwd<<<grid, kSsimThreads, 0, s>>>(img, tgt_rgb, depth, tgt_depth, tgt_depth ? depth_count : nullptr,
-                                                 view_weight, W, H, steps, t, lambda_ssim, cfg->lambda_depth, amap, bmap, cmap,
-                                                 dl_dimg, tgt_depth ? dl_ddepth : nullptr, acc, done, loss_view,
+                                                 view_weight, W, H, steps, t, lambda_ssim, cfg->lambda_depth, amap,
+                                                 bmap, cmap, dl_dimg, tgt_depth ? dl_ddepth : nullptr, acc, done, loss_view,
                                                  status_dev);
         e = cudaGetLastError();
     }

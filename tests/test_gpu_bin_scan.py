@@ -25,6 +25,8 @@ def length_class(lens):
     (1, 700, 512, 512, 8, 40),      # 4096: one whole block
     (1, 700, 514, 512, 8, 40),      # 4160: two blocks
     (3, 257, 512, 512, 8, 90),      # three blocks
+    (1, 300, 512, 512, 8, 34),      # rects around the 64 tiles of a mask
+    (1, 60, 512, 512, 8, 900),      # rects of the whole view: 32 runs of 128 tiles
     (1, 30000, 160, 120, 16, 9),    # chunks of 256
     (1, 60000, 160, 120, 16, 9),    # 512 on 152 SMs
     (2, 90000, 160, 120, 16, 9),    # 1024
