@@ -21,6 +21,19 @@ cudaError_t adam(float *p, const float *g, float *m, float *v, int64_t n, int de
                  cudaStream_t s);
 cudaError_t densify_stats(const float *rec, const float *sgrad, int64_t n, int V, const Grid &g, float *accum,
                           float *denom, float *maxr, int num_sms, cudaStream_t s);
+// Multiprocessors of the current device (queried once per device).
+int num_sms()
+{
+    static int cache[64] = {0};
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) return 132;
+    if (dev >= 0 && dev < 64 && cache[dev]) return cache[dev];
+    int v = 0;
+    if (cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || v <= 0) v = 132;
+    if (dev >= 0 && dev < 64) cache[dev] = v;
+    return v;
+}
+
 }  // namespace cgs
 
 using namespace cgs;
@@ -34,18 +47,6 @@ bool sizes_ok(int64_t n, int32_t V, const cgs_config *c)
     Grid g = make_grid(*c);
     if (g.Tv * V >= ((int64_t)1 << 31)) return false;
     return true;
-}
-
-int num_sms()
-{
-    static int cache[64] = {0};
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess) return 132;
-    if (dev >= 0 && dev < 64 && cache[dev]) return cache[dev];
-    int v = 0;
-    if (cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || v <= 0) v = 132;
-    if (dev >= 0 && dev < 64) cache[dev] = v;
-    return v;
 }
 
 int cuda_status(cudaError_t e)

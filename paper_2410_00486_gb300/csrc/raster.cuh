@@ -64,7 +64,7 @@ __device__ __forceinline__ void item_tile(const uint32_t *order, const Grid &g, 
 // the staged splat is read from shared memory once for PPT pixels and the backward's
 // per-(warp, splat) reduction covers 32*PPT pixels.
 // The forward keeps two (its per-thread state is small and occupancy pays; four measured
-// slower), the backward eight: one warp per 16x16 tile, half the warp reductions per pixel
+// slower; one on windows of few tiles), the backward eight: one warp per 16x16 tile, half the warp reductions per pixel
 // of four pixels, which were a third of its time (3.84 vs 4.04 ms on the 16-view window);
 // on windows of few tiles four or two, a part of the tile per warp.
 constexpr int kPPTFwd = 2;
@@ -165,6 +165,7 @@ __device__ __forceinline__ float staged_power(const float4 &t0, float hC, float 
     return power_at(power_x(t0, dx), hC, dy);
 }
 
+int num_sms();
 cudaError_t raster_fwd(const RasterFwdArgs &a, int B, int BD, cudaStream_t s);
 cudaError_t raster_bwd(const RasterBwdArgs &a, int B, int BD, int sms, cudaStream_t s);
 

@@ -1,12 +1,13 @@
 // Forward blend of Eq. 1 (Sec. III-B, CaRtGS) with the L1 loss fused in.
 //
-// One block per (view, tile), two pixels of one column per thread (4 rows apart).  The
-// tile's depth-sorted list (only splats that can reach alpha >= 1/255 in the tile: the
-// binning's test) is consumed in batches of BD splats: the block gathers the records of a
-// batch (48 bytes each, one per thread) into shared memory; every pixel then walks the
-// batch front to back, rejecting a pair on its base-2 exponent (|power| > -tau, both
-// scaled by log2 e) before any exponential.  A block-wide vote (__syncthreads_count) ends the walk
-// as soon as every pixel of the tile is saturated (T below 1e-4).
+// One block per (view, tile), two pixels of one column per thread (4 rows apart; one pixel on
+// windows of few tiles).  The tile's depth-sorted list (only splats that can reach alpha >=
+// 1/255 in the tile: the binning's test) is consumed in batches of BD splats: the block
+// gathers the records of a batch (48 bytes each, one per thread) into shared memory; every
+// pixel then walks the batch front to back, rejecting a pair on its base-2 exponent (|power| >
+// -tau, both scaled by log2 e) before any exponential.  A block-wide vote
+// (__syncthreads_count) ends the walk as soon as every pixel of the tile is saturated (T below
+// 1e-4).
 #include "raster.cuh"
 
 namespace cgs {
@@ -15,11 +16,10 @@ namespace cgs {
 // its exponent is NaN and it fails the alpha test with no branch of its own.
 __device__ constexpr float kNoRow = __builtin_nanf("");
 
-template <int B, int BD, bool CKPT, bool COUNT>
-__global__ void __launch_bounds__(B *B / ppt_for<B, kPPTFwd>(), (min_blocks_for<B, kPPTFwd, kFwdMinWarps>())) k_render_fwd(RasterFwdArgs a)
+template <int B, int BD, bool CKPT, bool COUNT, int PPT>
+__global__ void __launch_bounds__(B *B / PPT, (min_blocks_for<B, PPT, kFwdMinWarps>())) k_render_fwd(RasterFwdArgs a)
 {
     pdl_begin();   // the read-only loads below are addressed by what is read after the wait
-    constexpr int PPT = ppt_for<B, kPPTFwd>();
     constexpr int NT = B * B / PPT;
     constexpr int NW = NT / 32;
     __shared__ float4 s0[BD], s1[BD], s2[BD];
@@ -32,10 +32,11 @@ __global__ void __launch_bounds__(B *B / ppt_for<B, kPPTFwd>(), (min_blocks_for<
     // pixels covers 8 columns x 4 rows: a compact footprint, where fewer steps hold a
     // splat's edge, so fewer of a warp's lanes idle in the blend (1.721 -> 1.667 ms on the
     // 16-view window against 16 columns x 2 rows, images identical)
-    static_assert(PPT == 2 && NT * 2 == B * B, "two pixels per thread");
+    // With one pixel a thread (launch_fwd) a warp takes 8 columns x 4 rows.
+    static_assert(PPT == 1 || PPT == 2, "a thread's rows lie 4 apart");
     const int wq = (int)threadIdx.x >> 5, lq = (int)threadIdx.x & 31;
     const int col = 8 * (wq % (B / 8)) + (lq & 7);
-    const int row0 = 8 * (wq / (B / 8)) + (lq >> 3);
+    const int row0 = 4 * PPT * (wq / (B / 8)) + (lq >> 3);
     constexpr int G = 4;
     const int px = tx * B + col;
     const int py0 = ty * B + row0;   // row of pixel p: py0 + G p
@@ -232,17 +233,31 @@ k_loss_reduce(const float *__restrict__ partials, int64_t Tv, const float *__res
     }
 }
 
+// Two pixels a thread, or one on windows of at most kFwdWideTiles 16x16 tiles per SM: such a
+// window is bound by the walk of its longest lists, whose every step is shorter for one pixel,
+// a larger one by the issue of all its steps.  Measured (us, two pixels and one): 80 tiles
+// 15.6, 15.2; 300 tiles 17.8, 15.1; 475 tiles 22.1, 20.5; 1200 tiles 46.7, 35.5 (longer lists
+// 81, 62); 1900 tiles 53, 56; 2394 tiles 33, 39; 3600 tiles 92, 110; 9600 tiles 252, 298.
+constexpr int kFwdWideTiles = 8;
+
 template <int B, int BD>
 static cudaError_t launch_fwd(const RasterFwdArgs &a, cudaStream_t s)
 {
     const int64_t items = a.g.Tv * a.V;
-    const int nt = B * B / ppt_for<B, kPPTFwd>();
+    constexpr int P = ppt_for<B, kPPTFwd>();
+    const int nt = B * B / P;
+    if constexpr (B == 16) {
+        if (!a.ck4 && !a.count_blend && items <= kFwdWideTiles * (int64_t)num_sms()) {
+            launch(k_render_fwd<B, BD, false, false, 1>, (unsigned)items, B * B, 0, s, a);
+            return cudaGetLastError();
+        }
+    }
     if (a.ck4)   // the checkpointing forward does not count blended pairs
-        launch(k_render_fwd<B, BD, true, false>, (unsigned)items, nt, 0, s, a);
+        launch(k_render_fwd<B, BD, true, false, P>, (unsigned)items, nt, 0, s, a);
     else if (a.count_blend)
-        launch(k_render_fwd<B, BD, false, true>, (unsigned)items, nt, 0, s, a);
+        launch(k_render_fwd<B, BD, false, true, P>, (unsigned)items, nt, 0, s, a);
     else
-        launch(k_render_fwd<B, BD, false, false>, (unsigned)items, nt, 0, s, a);
+        launch(k_render_fwd<B, BD, false, false, P>, (unsigned)items, nt, 0, s, a);
     return cudaGetLastError();
 }
 
