@@ -31,9 +31,9 @@
 // as are resident on the GPU take (view, tile) items in the sort's longest-first order
 // from the counter until none is left.
 //
-// Windows of few tiles split each 16x16 tile into two or four parts (bwd_parts), a warp and
-// four or two pixels a thread each: one 160x120 view 44 -> 29 us, one 640x480 view of 40k
-// Gaussians 190 -> 127 us, three of 637x479 343 -> 280 us.
+// Windows of few tiles split each 16x16 tile into two or four parts, a warp and four or two
+// pixels a thread each, and the smallest its list into two segments (bwd_split): one 640x480
+// view of 40k Gaussians 190 -> 100 us, three of 637x479 343 -> 280 us.
 #include "raster.cuh"
 
 namespace cgs {
@@ -65,9 +65,12 @@ struct BwdSmem {
 
 // One work item: the tile at a place of the work order by NT threads of PPT pixels each, or
 // (S > 1) one of S parts of it by a warp on its own in a block of several: a half of eight
-// rows, or one of the four 8x8 blocks, whose short outline the fewest splats cross.
-template <int B, int BD, int NT, int PPT, int S, class Smem>
-__device__ __forceinline__ void bwd_item(const RasterBwdArgs &a, uint32_t place, int part, int tid, Smem &sm)
+// rows, or one of the four 8x8 blocks, whose short outline the fewest splats cross.  With SEG
+// > 1 an item is also one of SEG segments of the list: the splats behind its segment only
+// take the pixels' transmittance and colour behind to the segment's end, by the same steps
+// (the same bits) as the item that owns them.
+template <int B, int BD, int NT, int PPT, int S, int SEG, class Smem>
+__device__ __forceinline__ void bwd_item(const RasterBwdArgs &a, uint32_t place, int part, int seg, int tid, Smem &sm)
 {
     constexpr int NW = NT / 32;
     constexpr bool kWarp = S > 1, kBlocks = S == 4;
@@ -162,8 +165,11 @@ __device__ __forceinline__ void bwd_item(const RasterBwdArgs &a, uint32_t place,
             n2 = __ldg(r + 2);
         }
     };
+    const int seg0 = SEG > 1 ? (int)((uint64_t)maxlast * seg / SEG) : 0;
+    const int seg1 = SEG > 1 ? (int)((uint64_t)maxlast * (seg + 1) / SEG) : (int)maxlast;
+    if (SEG > 1 && seg0 == seg1) return;   // item-uniform
     if (kAhead) fetch((int)maxlast);
-    for (int bend = (int)maxlast; bend > 0; bend -= BD) {
+    for (int bend = (int)maxlast; bend > seg0; bend -= BD) {
         const int bstart = kAhead ? bend - BD : max(0, bend - BD);   // below 0: the batch's first lanes are empty
         const int nraw = bend - bstart;
         item_sync();
@@ -188,11 +194,31 @@ __device__ __forceinline__ void bwd_item(const RasterBwdArgs &a, uint32_t place,
             }
         }
         item_sync();
-        const int j0 = kAhead ? max(0, -bstart) : 0;
+        const int j0 = kAhead ? max(0, seg0 - bstart) : 0;
+        int jtop = nraw - 1;
+        if (SEG > 1) {
+            // behind the segment: transmittance and colour behind only
+#pragma unroll 4
+            for (; jtop >= max(j0, seg1 - bstart); jtop--) {
+                const uint32_t pos = (uint32_t)(bstart + jtop);
+                const float4 q0 = s0[jtop], q1 = s1[jtop], q2 = s2[jtop];
+                const PowerX pxs = power_x(q0, __fsub_rn(q0.x, fx));
+#pragma unroll
+                for (int p = 0; p < PPT; p++) {
+                    const float pw = power_at(pxs, q1.x, __fsub_rn(q0.y, fy0 + (float)(G * p)));
+                    if (!(pos < lst[p] && fabsf(pw) <= q1.w)) continue;
+                    const float4 gi = sgi[p * NT + tid];
+                    const float alpha = fminf(kAlphaMax, __fmul_rn(q1.y, exp2_fast(pw)));
+                    T[p] = T[p] * rcp_fast(__fsub_rn(1.f, alpha));
+                    const float cg = fmaf(q1.z, gi.w, fmaf(q2.z, gi.z, fmaf(q2.y, gi.y, q2.x * gi.x)));
+                    Sb[p] = fmaf(alpha, cg - Sb[p], Sb[p]);
+                }
+            }
+        }
         // two splats per loop trip, so one splat's loads and tests overlap the other's blend and
         // sums (3.470 -> 3.426 ms on the 16-view window; four per trip spill: 3.87 ms)
 #pragma unroll 2
-        for (int j = nraw - 1; j >= j0; j--) {
+        for (int j = jtop; j >= j0; j--) {
             const uint32_t pos = (uint32_t)(bstart + j);   // list position of splat j
             const float4 q0 = s0[j];
             const float4 q1 = s1[j];
@@ -351,14 +377,14 @@ __global__ void __launch_bounds__(B *B / ppt_for<B, kPPTBwd>(), (min_blocks_for<
         } else if (it > 0) {
             break;
         }
-        bwd_item<B, BD, NT, PPT, 1>(a, item, 0, threadIdx.x, sm);
+        bwd_item<B, BD, NT, PPT, 1, 1>(a, item, 0, 0, threadIdx.x, sm);
     }
 }
 
-// Windows of few 16x16 tiles (bwd_parts): the warps of a block of four take parts of tiles,
+// Windows of few 16x16 tiles (bwd_split): the warps of a block of four take parts of tiles,
 // each on its own.
 constexpr int kPartWarps = 4, kPartMinBlocks = 5;
-template <int S>
+template <int S, int SEG>
 __global__ void __launch_bounds__(32 * kPartWarps, kPartMinBlocks) k_render_bwd_parts(RasterBwdArgs a)
 {
     pdl_begin();   // the read-only loads below are addressed by what is read after the wait
@@ -366,7 +392,7 @@ __global__ void __launch_bounds__(32 * kPartWarps, kPartMinBlocks) k_render_bwd_
     auto &sm = smem[threadIdx.x >> 5];
     const int lane = threadIdx.x & 31;
     zero_rows(sm.red, lane, 32);
-    const uint32_t n_items = (uint32_t)(a.g.Tv * a.V) * S;
+    const uint32_t n_items = (uint32_t)(a.g.Tv * a.V) * (S * SEG);
     for (uint32_t it = 0;; it++) {
         uint32_t item = blockIdx.x * kPartWarps + (threadIdx.x >> 5);
         __syncwarp();   // the zero rows are written; the previous item's reads of the shared state are done
@@ -377,20 +403,29 @@ __global__ void __launch_bounds__(32 * kPartWarps, kPartMinBlocks) k_render_bwd_
             break;
         }
         if (item >= n_items) break;
-        bwd_item<16, 32, 32, 8 / S, S>(a, item / S, (int)(item % S), lane, sm);
+        bwd_item<16, 32, 32, 8 / S, S, SEG>(a, item / (S * SEG), (int)(item / SEG % S), (int)(item % SEG), lane, sm);
     }
 }
 
-// Parts of a tile.  With one part the warp sums cover most pixels, which is best when the
-// window has work for the whole GPU; a window of few tiles is bound by the walk of its longest
-// list, one warp's chain of dependent steps, each shorter the fewer pixels the warp blends.
-// Measured (us, one, two and four parts): 80 tiles 52, 38, 29; 1200 tiles 193, 148, 127; 1900
-// tiles 242, 199, 166; 2394 tiles 142, 112, 110; 3225 tiles 321, 278, 335; 3600 tiles 386, 280,
-// 327; 5700 tiles 494, 524, 633; 9600 tiles 756, 838, 966.  Splitting only the longest lists'
-// tiles in four: 3225 tiles 314 to 395, 5700 tiles 493 to 602, never the best.
-static int bwd_parts(int64_t tiles, int sms)
+// Parts of a tile and segments of its list.  With one of each the warp sums cover most pixels,
+// which is best when the window has work for the whole GPU; a window of few tiles is bound by
+// the walk of its longest list, one warp's chain of dependent steps, each shorter the fewer
+// pixels the warp blends, and fewer with the list in segments.
+// Measured together with the projection's backward (us; one, two and four parts,
+// four parts in two and in four segments): 80 tiles 49, 34, 27, 23, 23; 300 tiles 67, 45, 37,
+// 34, 36; 475 tiles 97, 68, 57, 49, 44; 1200 tiles 193, 146, 128, 105, 132; with longer lists
+// 312, 233, 200, 194, 238; 1900 tiles 237, 194, 164, 193, 247; 2394 tiles 135, 111, 109, 131,
+// 173; 3225 tiles 307, 276, 333; 3600 tiles 365, 275, 325; 5700 tiles 464, 521, 632; 9600 tiles
+// 767, 833, 966.  Two parts in two segments: 158 at 1900 tiles, 106 at 2394, else slower.
+// Splitting only the longest lists' tiles: 3225 tiles 314 to 395, 5700 tiles 493 to 602.
+struct BwdSplit {
+    int parts, segments;
+};
+static BwdSplit bwd_split(int64_t tiles, int sms)
 {
-    return tiles <= 16 * (int64_t)sms ? 4 : (tiles <= 32 * (int64_t)sms ? 2 : 1);
+    if (tiles <= 8 * (int64_t)sms) return BwdSplit{4, 2};
+    if (tiles <= 16 * (int64_t)sms) return BwdSplit{4, 1};
+    return BwdSplit{tiles <= 32 * (int64_t)sms ? 2 : 1, 1};
 }
 
 // Blocks of a persistent launch: as many as are resident on the GPU (queried once per device
@@ -427,16 +462,16 @@ static cudaError_t launch_bwd(const RasterBwdArgs &a, int sms, cudaStream_t s)
     return cudaGetLastError();
 }
 
-template <int S>
+template <int S, int SEG>
 static cudaError_t launch_bwd_parts(const RasterBwdArgs &a, int sms, cudaStream_t s)
 {
-    int64_t blocks = (a.g.Tv * a.V * S + kPartWarps - 1) / kPartWarps;
+    int64_t blocks = (a.g.Tv * a.V * (S * SEG) + kPartWarps - 1) / kPartWarps;
     if (a.work) {
         static int resident[64] = {0};
-        const cudaError_t e = persistent_blocks(a, k_render_bwd_parts<S>, 32 * kPartWarps, resident, sms, blocks, s);
+        const cudaError_t e = persistent_blocks(a, k_render_bwd_parts<S, SEG>, 32 * kPartWarps, resident, sms, blocks, s);
         if (e != cudaSuccess) return e;
     }
-    launch(k_render_bwd_parts<S>, (unsigned)blocks, 32 * kPartWarps, 0, s, a);
+    launch(k_render_bwd_parts<S, SEG>, (unsigned)blocks, 32 * kPartWarps, 0, s, a);
     return cudaGetLastError();
 }
 
@@ -444,9 +479,10 @@ template <int B>
 static cudaError_t launch_bwd_bd(const RasterBwdArgs &a, int BD, int sms, cudaStream_t s)
 {
     if (B == 16) {
-        const int parts = bwd_parts(a.g.Tv * a.V, sms);
-        if (parts == 4) return launch_bwd_parts<4>(a, sms, s);
-        if (parts == 2) return launch_bwd_parts<2>(a, sms, s);
+        const BwdSplit split = bwd_split(a.g.Tv * a.V, sms);
+        if (split.parts == 4 && split.segments == 2) return launch_bwd_parts<4, 2>(a, sms, s);
+        if (split.parts == 4) return launch_bwd_parts<4, 1>(a, sms, s);
+        if (split.parts == 2) return launch_bwd_parts<2, 1>(a, sms, s);
     }
     switch (BD) {
     case 32: return launch_bwd<B, 32>(a, sms, s);

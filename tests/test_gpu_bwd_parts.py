@@ -1,5 +1,6 @@
 """The raster backward on both sides of the tile counts where it goes from four parts of a
-tile to two and to whole tiles (16 and 32 tiles per SM), against the oracle's."""
+tile in two list segments to whole lists, to two parts and to whole tiles (8, 16 and 32 tiles
+per SM), against the oracle's."""
 from __future__ import annotations
 
 import numpy as np
@@ -14,7 +15,7 @@ from test_gpu_parity import (gpu_forward_from_rec, residual_sign_flags, round32,
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("W,H,views", [(16, 16, 1), (33, 47, 3), (1024, 608, 1), (1023, 624, 1), (1216, 1023, 1),
+@pytest.mark.parametrize("W,H,views", [(16, 16, 1), (33, 47, 3), (608, 512, 1), (609, 511, 1), (1024, 608, 1), (1023, 624, 1), (1216, 1023, 1),
                                        (1216, 1040, 1)])
 @pytest.mark.parametrize("persistent", [True, False])
 def test_raster_bwd_parts(W, H, views, persistent):
