@@ -113,10 +113,13 @@ static int64_t chunk_count_entries(int64_t n, int64_t V, int64_t Tv, int chunk)
     return (n + chunk - 1) / chunk * V * Tv;
 }
 
+// Bytes for every chunk size that n or fewer Gaussians may take: chunks below kChunkSmall come
+// to at most 2 num_sms blocks, so a workspace kept for a growing map also serves a smaller one.
 size_t bin_ws_bytes(int64_t capacity, int64_t n, int64_t V, int64_t Tv, int num_sms)
 {
-    return ws_layout(capacity, Tv * V, chunk_count_entries(n, V, Tv, chunk_for(n, V, num_sms)), V * n, nullptr,
-                     nullptr);
+    int64_t counts = chunk_count_entries(n, V, Tv, chunk_for(n, V, num_sms));
+    if (counts > 0) counts = std::max(counts, std::min((n + kChunkMin - 1) / kChunkMin * V, 2 * (int64_t)num_sms) * Tv);
+    return ws_layout(capacity, Tv * V, counts, V * n, nullptr, nullptr);
 }
 
 __device__ __forceinline__ bool load_slot(const float4 *__restrict__ rec, int64_t slot, float &u, float &v,
