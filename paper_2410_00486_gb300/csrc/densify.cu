@@ -235,7 +235,7 @@ k_densify_apply(const float *__restrict__ P, const float *__restrict__ Mi, const
 // is one contiguous run of points.  Per point a search over growing rings of cells stops
 // once the distance to the unsearched region, less a rounding margin, is at least the
 // third-best distance (k_knn); points not settled within kNearRings rings are listed and
-// searched by a block each (k_knn_far).
+// searched by a block each (knn_far).
 
 constexpr int kGridCap = 128;
 constexpr int kKnn = 3;
@@ -243,9 +243,9 @@ constexpr float kKnnFloor = 1e-7f;
 constexpr float kShC0 = 0.28209479177387814f;
 // Rings a single thread searches.  A stray point far outside the room has to look at
 // every cell of the grid: one thread walking them alone took 122 ms on a 307k-point frame
-// with two such points, where k_knn takes 160 us and k_knn_far 17 us.
+// with two such points, where k_knn takes 160 us and a block for each of the two 17 us.
 constexpr int kNearRings = 4;
-constexpr int kFarThreads = 512, kFarSample = 4096;
+constexpr int kFarThreads = 512, kFarBlocks = 304, kFarSample = 4096;
 
 struct GridInfo {
     float lo[3];
@@ -254,7 +254,7 @@ struct GridInfo {
     float margin;
     uint32_t box[6];   // sortable encodings, all maxima: complements of min x, y, z, then max x, y, z
     uint32_t done;     // blocks of k_bbox that have added their part
-    uint32_t nfar;     // points listed for k_knn_far
+    uint32_t nfar;     // points listed for knn_far
     double sum[3], sumsq[3];
 };
 
@@ -535,12 +535,12 @@ k_knn(const float4 *__restrict__ pts, int64_t m, GridInfo *__restrict__ gi, cons
     }
 }
 
-// The listed points, one block each.  An evenly spaced sample of the cloud bounds the
-// third-best distance first; then the lanes of a warp take 32 rows of cells at a time, cut to
-// the cells within that distance, and those rows' points together.
-__global__ void __launch_bounds__(kFarThreads)
-k_knn_far(const float4 *__restrict__ pts, int64_t m, const GridInfo *__restrict__ gi,
-          const uint32_t *__restrict__ off, const uint32_t *__restrict__ far, float *__restrict__ ls)
+// The listed points, one block each (of `blocks`).  An evenly spaced sample of the cloud
+// bounds the third-best distance first; then the lanes of a warp take 32 rows of cells at a
+// time, cut to the cells within that distance, and those rows' points together.
+__device__ __forceinline__ void knn_far(uint32_t block, uint32_t blocks, const float4 *__restrict__ pts, int64_t m,
+                                        const GridInfo *__restrict__ gi, const uint32_t *__restrict__ off,
+                                        const uint32_t *__restrict__ far, float *__restrict__ ls)
 {
     constexpr int NW = kFarThreads / 32;
     __shared__ Best sbest[NW];
@@ -567,7 +567,7 @@ k_knn_far(const float4 *__restrict__ pts, int64_t m, const GridInfo *__restrict_
         return best;
     };
     const uint32_t nfar = gi->nfar;
-    for (uint32_t f = blockIdx.x; f < nfar; f += gridDim.x) {
+    for (uint32_t f = block; f < nfar; f += blocks) {
         const uint32_t t = far[f];
         const float4 me = pts[t];
         const Query Q(*gi, me, t, m);
@@ -632,19 +632,19 @@ struct Run {
     float value;
     int kind;
 };
-constexpr int kMaxRuns = 36, kRunThreads = 256, kRunChunk = 16 * kRunThreads;
+constexpr int kMaxRuns = 36, kRunThreads = kFarThreads, kRunChunk = 16 * kRunThreads;
 struct Runs {
     Run run[kMaxRuns];
     int n;
     int64_t blocks;
 };
 
-__global__ void __launch_bounds__(kRunThreads) k_runs(const __grid_constant__ Runs R)
+__device__ __forceinline__ void fill_run(const Runs &R, int64_t block)
 {
     int k = 0;
-    while (k + 1 < R.n && (int64_t)blockIdx.x >= R.run[k + 1].block0) k++;
+    while (k + 1 < R.n && block >= R.run[k + 1].block0) k++;
     const Run &r = R.run[k];
-    const int64_t e0 = (blockIdx.x - r.block0) * kRunChunk;
+    const int64_t e0 = (block - r.block0) * kRunChunk;
     const int cnt = (int)min((int64_t)kRunChunk, r.len - e0);
     float *d = r.dst + e0;
     const float *s = r.src ? r.src + e0 : nullptr;
@@ -681,6 +681,21 @@ __global__ void __launch_bounds__(kRunThreads) k_runs(const __grid_constant__ Ru
     }
 }
 static_assert(kRunChunk % 4 == 0, "a chunk of quaternions starts at a whole one");
+
+__global__ void __launch_bounds__(kRunThreads) k_runs(const __grid_constant__ Runs R) { fill_run(R, blockIdx.x); }
+
+// The far points' search beside the runs: a few blocks waiting on memory, hidden by the copies
+// (17 us of a 307k-point frame with two strays).
+__global__ void __launch_bounds__(kFarThreads)
+k_far_runs(const __grid_constant__ Runs R, const float4 *__restrict__ pts, int64_t m,
+           const GridInfo *__restrict__ gi, const uint32_t *__restrict__ off, const uint32_t *__restrict__ far,
+           float *__restrict__ ls)
+{
+    if (blockIdx.x < kFarBlocks)
+        knn_far(blockIdx.x, kFarBlocks, pts, m, gi, off, far, ls);
+    else
+        fill_run(R, (int64_t)blockIdx.x - kFarBlocks);
+}
 
 static void add_run(Runs &R, float *dst, const float *src, int64_t len, int kind, float value = 0.f)
 {
@@ -809,9 +824,11 @@ int cgs_points_to_gaussians(const float *params, const float *m, const float *v,
     }
     if (n_points > 0 && ((uintptr_t)workspace & 255) != 0) return CGS_ERR_ARG;
     if (n_points > 0 && workspace_bytes < cgs_points_workspace(n_points)) return CGS_ERR_WORKSPACE;
-    if (R.blocks >= (int64_t)1 << 31) return CGS_ERR_ARG;
-    k_runs<<<(unsigned)R.blocks, kRunThreads, 0, s>>>(R);
-    if (n_points == 0) return st_of(cudaGetLastError());
+    if (R.blocks + kFarBlocks >= (int64_t)1 << 31) return CGS_ERR_ARG;
+    if (n_points == 0) {
+        k_runs<<<(unsigned)R.blocks, kRunThreads, 0, s>>>(R);
+        return st_of(cudaGetLastError());
+    }
     const int64_t B = grid_cell_budget(n_points);
     char *w = static_cast<char *>(workspace);
     GridInfo *gi = reinterpret_cast<GridInfo *>(w);
@@ -840,7 +857,7 @@ int cgs_points_to_gaussians(const float *params, const float *m, const float *v,
     const int kb = (int)((n_points + 127) / 128 < 8192 ? (n_points + 127) / 128 : 8192);
     float *ls = params_out + 3 * n_out + 3 * n;   // log-scales of the new Gaussians
     k_knn<<<kb, 128, 0, s>>>(pts, n_points, gi, off, cell_of, ls);
-    k_knn_far<<<304, kFarThreads, 0, s>>>(pts, n_points, gi, off, cell_of, ls);
+    k_far_runs<<<(unsigned)(kFarBlocks + R.blocks), kFarThreads, 0, s>>>(R, pts, n_points, gi, off, cell_of, ls);
     return st_of(cudaGetLastError());
 }
 
