@@ -442,11 +442,11 @@ def main():
     st = win.read_status()
     if st[0] != 0:
         raise SystemExit(f"device status after timing: {st}")
-    # preprocess, count, scan x2 (with the work order; one launch up to 4096 tiles), scatter, sort x3 (lists
-    # above 1024 and above 2048 entries only where a view has that many Gaussians), fwd, loss reduce, raster
-    # bwd, preprocess bwd, adam, step counter (the launch list of the captured 16-view iteration shows these
-    # 14 kernels per step)
-    launches_per_step = 14 - (win.Ttot <= 4096) - (sc.n <= 1024) - (sc.n <= 2048)
+    # preprocess, clear of the counters, count, scan x2 (with the work order; one launch up to 4096 tiles),
+    # scatter, sort x3 (lists above 1024 and above 2048 entries only where a view has that many Gaussians),
+    # fwd, loss reduce, clear of the work counter, raster bwd, preprocess bwd, step counter, adam (the launch
+    # list of the captured 16-view iteration shows these 16 kernels per step)
+    launches_per_step = 16 - (win.Ttot <= 4096) - (sc.n <= 1024) - (sc.n <= 2048)
     gpu_launches = args.steps * launches_per_step
     clocks = clk.summary()
     k_forms = max(MIN_FORM_STEPS, args.steps)

@@ -1159,7 +1159,7 @@ cudaError_t bin_sort(const float *rec, int64_t n, int V, const Grid &g, void *ws
     const int chunk = chunk_for(n, V, num_sms);
     ws_layout(capacity, Ttot, chunk_count_entries(n, V, g.Tv, chunk), (int64_t)V * n, &w, ws);
     const float4 *r4 = reinterpret_cast<const float4 *>(rec);
-    cudaError_t e = cudaMemsetAsync(w.count, 0, sizeof(uint32_t) * (2 * (size_t)Ttot + 3), s);
+    cudaError_t e = clear_words(w.count, 2 * Ttot + 3, s);
     if (e != cudaSuccess) return e;
     const int64_t slots = (int64_t)V * n;
     const size_t hist_bytes = sizeof(uint32_t) * (size_t)g.Tv;

@@ -74,6 +74,21 @@ inline cudaError_t launch(void (*kernel)(K...), dim3 grid, dim3 block, size_t sm
     return cudaLaunchKernelEx(&cfg, kernel, std::forward<A>(args)...);
 }
 
+// Zeroes n words in the chain of dependent launches, which a memset would break (two in an
+// iteration: one 160x120 view 59.4 -> 50.3 us, one 640x480 view 181 -> 176).
+template <class T>
+__global__ void k_clear(T *p, int64_t n)
+{
+    pdl_begin(p);
+    const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (i < n) p[i] = T(0);
+}
+template <class T>
+inline cudaError_t clear_words(T *p, int64_t n, cudaStream_t s)
+{
+    return launch(k_clear<T>, (unsigned)((n + 255) / 256), 256, 0, s, p, n);
+}
+
 // Record a device-side condition; the first one wins.
 __device__ __forceinline__ void set_status(int32_t *st, int code)
 {

@@ -445,7 +445,7 @@ static cudaError_t persistent_blocks(const RasterBwdArgs &a, K kernel, int threa
         resident[dev] = max(1, per_sm) * max(1, sms);
     }
     blocks = min(blocks, (int64_t)resident[dev]);
-    return cudaMemsetAsync(a.work, 0, sizeof(uint32_t), s);
+    return clear_words(a.work, 1, s);
 }
 
 template <int B, int BD>
