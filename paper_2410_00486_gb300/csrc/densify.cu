@@ -145,9 +145,11 @@ k_densify_plan(const float *__restrict__ P, int64_t n, int64_t span, const float
 // shared memory says which Gaussian each output copies, and every group is then written
 // as one contiguous run of floats, lanes along it, so stores are whole lines and loads
 // nearly so (the copies of a Gaussian repeat its floats, a pruned one leaves a gap).  Bound
-// by HBM: 200k Gaussians of SH degree 3 in 78 us, 3.7 TB/s; one thread per Gaussian,
-// copying it float by float with the rows of a warp 180 bytes apart, took 266 us.
-constexpr int kDenG = 128, kDenThreads = 256;
+// by HBM and its latency: 200k Gaussians of SH degree 3 in 61 us, 4.7 TB/s; one thread per
+// Gaussian, copying it float by float with the rows of a warp 180 bytes apart, took 266 us,
+// the groups one after another and a load and a store at a time 78.  Eight floats ahead, or
+// blocks of 64 Gaussians, measure the same.
+constexpr int kDenG = 128, kDenThreads = 256, kDenAhead = 4;
 constexpr uint16_t kDenFresh = 0x4000, kDenSplit = 0x8000;   // zero moments; mean and scale drawn anew
 
 template <int DEG>
@@ -196,24 +198,44 @@ k_densify_apply(const float *__restrict__ P, const float *__restrict__ Mi, const
         }
     }
     __syncthreads();
+    // the groups side by side: a warp for means and scales, one for rotations, opacities and
+    // DC colours, the others for the higher bands, so no group waits for another's loads,
+    // and a thread's kDenAhead floats of each array on their way together
     const int outs = s_outs;
+    const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
     const int widths[6] = {3, 3, 4, 1, 3, R3};
     int64_t oi = 0, oo = 0;
 #pragma unroll
     for (int gi = 0; gi < 6; gi++) {
         const int w = widths[gi];
         if (w == 0) continue;
-        const float *pi = P + oi + w * g0, *mi = Mi + oi + w * g0, *vi = Vi + oi + w * g0;
-        float *po = Po + oo + w * j0, *mo = Mo + oo + w * j0, *vo = Vo + oo + w * j0;
-#pragma unroll 4
-        for (int i = threadIdx.x; i < w * outs; i += kDenThreads) {
-            const int jl = i / w;
-            const uint32_t e = src[jl];
-            const int from = w * (int)(e & (kDenFresh - 1)) + i - w * jl;
-            const bool fresh = e & kDenFresh;
-            if (gi >= 2 || !(e & kDenSplit)) po[i] = __ldg(pi + from);
-            mo[i] = fresh ? 0.f : __ldg(mi + from);
-            vo[i] = fresh ? 0.f : __ldg(vi + from);
+        const bool mine = gi < 2 ? wp == 0 : (gi < 5 ? wp == 1 : wp >= 2);   // warp-uniform
+        if (mine) {
+            const float *pi = P + oi + w * g0, *mi = Mi + oi + w * g0, *vi = Vi + oi + w * g0;
+            float *po = Po + oo + w * j0, *mo = Mo + oo + w * j0, *vo = Vo + oo + w * j0;
+            const int first = gi < 5 ? lane : lane + 32 * (wp - 2), step = gi < 5 ? 32 : kDenThreads - 64;
+            for (int i0 = first; i0 < w * outs; i0 += kDenAhead * step) {
+                float x[kDenAhead], y[kDenAhead], z[kDenAhead];   // every load before the first store
+                uint32_t e[kDenAhead];
+#pragma unroll
+                for (int q = 0; q < kDenAhead; q++) {
+                    const int i = i0 + q * step, jl = i / w;
+                    const bool in = i < w * outs;
+                    e[q] = in ? src[jl] : kDenFresh;
+                    const int from = w * (int)(e[q] & (kDenFresh - 1)) + i - w * jl;
+                    x[q] = in ? __ldg(pi + from) : 0.f;
+                    y[q] = e[q] & kDenFresh ? 0.f : __ldg(mi + from);
+                    z[q] = e[q] & kDenFresh ? 0.f : __ldg(vi + from);
+                }
+#pragma unroll
+                for (int q = 0; q < kDenAhead; q++) {
+                    const int i = i0 + q * step;
+                    if (i >= w * outs) break;
+                    if (gi >= 2 || !(e[q] & kDenSplit)) po[i] = x[q];
+                    mo[i] = y[q];
+                    vo[i] = z[q];
+                }
+            }
         }
         oi += (int64_t)w * n;
         oo += (int64_t)w * m;
