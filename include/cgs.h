@@ -226,9 +226,10 @@ int cgs_render_fwd_noalloc(const float *rec, const uint32_t *vals, const uint32_
  * from the caller (dl_dimg float[V][3][H][W], dl_ddepth float[V][H][W] or NULL).
  *   slot_grad  device in/out: accumulated (+=); zeroed by cgs_preprocess
  *   work       device uint32[1] or NULL.  Given, the launch is persistent: as many blocks as
- *              the GPU holds resident take the (view, tile) items, in tile_order, from this
- *              counter (the call sets it to 0 first and leaves the number of items taken plus
- *              the blocks in it).  NULL: one block per item.  Results are the same either way
+ *              the GPU holds resident take the (view, tile) items, or in windows of few tiles
+ *              parts of them, in tile_order, from this counter (the call sets it to 0 first
+ *              and leaves in it the number of items taken plus one for every taker that found
+ *              none left).  NULL: every item is launched.  Results are the same either way
  *              up to float summation order; calls that share a counter must not overlap.
  */
 int cgs_raster_bwd(const float *rec, const uint32_t *vals, const uint32_t *ranges,
@@ -368,7 +369,7 @@ int cgs_densify_apply(const float *params, const float *m, const float *v, int64
  * params / m / v (NULL allowed when n = 0), then point i as Gaussian n + i with zero Adam
  * moments.  xyz, rgb: device float[n_points][3].  The workspace (cgs_points_workspace(n_points)
  * bytes, 256-byte aligned) holds a uniform grid of the points' bounding box (about one cell
- * per point of its volume, at most 128 cells per axis) and the point ids sorted by cell.
+ * per point of its volume, at most 128 cells per axis) and the points sorted by cell.
  * Outputs must not alias inputs.  A non-finite coordinate sets CGS_ERR_NONFINITE in
  * *status_dev (that point's outputs are then unspecified).
  */

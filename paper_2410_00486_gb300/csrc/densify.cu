@@ -166,6 +166,7 @@ k_densify_apply(const float *__restrict__ P, const float *__restrict__ Mi, const
     const int cnt = (int)min((int64_t)kDenG, n - g0);
     const int64_t j0 = off[g0];
     if (threadIdx.x == 0) s_outs = 0;
+    for (int i = threadIdx.x; i < 2 * kDenG; i += kDenThreads) src[i] = kDenFresh;   // whatever the workspace holds
     __syncthreads();
     for (int gl = threadIdx.x; gl < cnt; gl += kDenThreads) {
         const int64_t g = g0 + gl, j = off[g];
