@@ -98,7 +98,7 @@ __global__ void __launch_bounds__(256) k_adam_vec(AdamArgs a)
     float4 p = make_float4(0.f, 0.f, 0.f, 0.f), g = p, m = p, v = p;
     auto load = [&] {
         p = p4[q];
-        g = __ldg(g4 + q);
+        g = g4[q];
         m = m4[q];
         v = v4[q];
     };
@@ -195,16 +195,16 @@ cudaError_t adam(float *p, const float *g, float *m, float *v, int64_t n, int de
 }
 
 __global__ void __launch_bounds__(256)
-k_densify(const float4 *__restrict__ rec, const float4 *__restrict__ sgrad, int64_t n, int V, float halfW, float halfH,
+k_densify(const float4 *rec, const float4 *sgrad, int64_t n, int V, float halfW, float halfH,
           float *__restrict__ accum, float *__restrict__ denom, float *__restrict__ maxr)
 {
     pdl_begin(rec, sgrad, accum, denom, maxr);
     const int64_t total = (int64_t)V * n;
     for (int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; s < total; s += (int64_t)gridDim.x * blockDim.x) {
-        const int r = __float_as_int(__ldg(reinterpret_cast<const float *>(rec + kRec4 * s) + 7));
+        const int r = __float_as_int(reinterpret_cast<const float *>(rec + kRec4 * s)[7]);
         if (r <= 0) continue;
         const int64_t g = s % n;
-        const float4 G = __ldg(sgrad + kRec4 * s);
+        const float4 G = sgrad[kRec4 * s];
         const float gx = G.x * halfW, gy = G.y * halfH;
         atomicAdd(accum + g, sqrtf(gx * gx + gy * gy));
         atomicAdd(denom + g, 1.0f);

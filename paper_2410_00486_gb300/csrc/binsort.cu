@@ -122,26 +122,25 @@ size_t bin_ws_bytes(int64_t capacity, int64_t n, int64_t V, int64_t Tv, int num_
     return ws_layout(capacity, Tv * V, counts, V * n, nullptr, nullptr);
 }
 
-__device__ __forceinline__ bool load_slot(const float4 *__restrict__ rec, int64_t slot, float &u, float &v,
-                                          float &z, int &r)
+__device__ __forceinline__ bool load_slot(const float4 *rec, int64_t slot, float &u, float &v, float &z, int &r)
 {
     const float *rf = reinterpret_cast<const float *>(rec + kRec4 * slot);
-    r = __float_as_int(__ldg(rf + 7));
+    r = __float_as_int(rf[7]);
     if (r <= 0) return false;
-    float4 a = __ldg(rec + kRec4 * slot);
+    float4 a = rec[kRec4 * slot];
     u = a.x;
     v = a.y;
-    z = __ldg(rf + 6);
+    z = rf[6];
     return true;
 }
 
 // The per-slot part of the tile reach test (record fields 2, 3, 4: conic; 11: tau).  With
 // rect lists every tile of the rect is kept (mode 1, "reaches everything").
-__device__ __forceinline__ ReachPre load_reach(const float4 *__restrict__ rec, int64_t slot, const Grid &g)
+__device__ __forceinline__ ReachPre load_reach(const float4 *rec, int64_t slot, const Grid &g)
 {
     if (g.rect_lists) return ReachPre{0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 1};
     const float *rf = reinterpret_cast<const float *>(rec + kRec4 * slot);
-    return reach_prepare(__ldg(rf + 2), __ldg(rf + 3), __ldg(rf + 4), __ldg(rf + 11));
+    return reach_prepare(rf[2], rf[3], rf[4], rf[11]);
 }
 
 // Does the slot (centre u, v) belong in tile (tx, ty): can it reach alpha >= 1/255 there?
@@ -152,7 +151,7 @@ __device__ __forceinline__ bool in_tile(const ReachPre &e, float u, float v, int
     return reach_box(e, u, v, bx0, bx1, by0, by1);
 }
 
-__global__ void k_count(const float4 *__restrict__ rec, int64_t n, int V, Grid g, uint32_t *__restrict__ count)
+__global__ void k_count(const float4 *rec, int64_t n, int V, Grid g, uint32_t *__restrict__ count)
 {
     pdl_begin(rec, count);
     const int64_t total = (int64_t)V * n;
@@ -277,7 +276,7 @@ __device__ __forceinline__ void rect_tile(int idx, int w, float inv, int &row, i
 }
 
 // A visible slot's reach test and the tiles it may reach (none: T empty).
-__device__ __forceinline__ bool slot_reach(const float4 *__restrict__ rec, int64_t slot, const Grid &g, float &u,
+__device__ __forceinline__ bool slot_reach(const float4 *rec, int64_t slot, const Grid &g, float &u,
                                            float &v, uint32_t &zb, ReachPre &e, Rect &T)
 {
     float z;
@@ -292,7 +291,7 @@ __device__ __forceinline__ bool slot_reach(const float4 *__restrict__ rec, int64
 }
 
 template <bool RECORD, class F>
-__device__ __forceinline__ void for_each_tile_pair(const float4 *__restrict__ rec, int64_t n, int view, int64_t s0,
+__device__ __forceinline__ void for_each_tile_pair(const float4 *rec, int64_t n, int view, int64_t s0,
                                                    int64_t s1, const Grid &g, uint32_t *next, LargeList &large,
                                                    PairStage &st, uint4 *__restrict__ slotrec, F f)
 {
@@ -441,7 +440,7 @@ constexpr int kAggWarps = kAggThreads / 32;
 constexpr size_t kStageBytes = sizeof(PairStage) * kAggWarps;
 
 __global__ void __launch_bounds__(kAggThreads, kAggMinBlocks)
-k_count_agg(const float4 *__restrict__ rec, int64_t n, int chunk, Grid g, uint32_t *__restrict__ count,
+k_count_agg(const float4 *rec, int64_t n, int chunk, Grid g, uint32_t *__restrict__ count,
             uint32_t *__restrict__ bcount, uint4 *__restrict__ slotrec)
 {
     pdl_begin(rec, count, bcount, slotrec);
@@ -480,7 +479,7 @@ __device__ __forceinline__ uint32_t len_bucket(uint32_t len)
 }
 
 __global__ void __launch_bounds__(kScanThreads)
-k_scan_part(const uint32_t *__restrict__ count, int64_t Ttot, unsigned long long *__restrict__ part,
+k_scan_part(const uint32_t *count, int64_t Ttot, unsigned long long *__restrict__ part,
             uint32_t *__restrict__ bhist)
 {
     pdl_begin(count, part, bhist);
@@ -522,8 +521,8 @@ k_scan_part(const uint32_t *__restrict__ count, int64_t Ttot, unsigned long long
 // 160x120: 11.7 and 4.3).
 template <bool ONE>
 __global__ void __launch_bounds__(kScanThreads)
-k_scan_out(uint32_t *__restrict__ count, int64_t Ttot, int64_t capacity, const unsigned long long *__restrict__ part,
-           const uint32_t *__restrict__ bhist, int nblocks, uint32_t *__restrict__ ranges,
+k_scan_out(uint32_t *__restrict__ count, int64_t Ttot, int64_t capacity, const unsigned long long *part,
+           const uint32_t *bhist, int nblocks, uint32_t *__restrict__ ranges,
            uint32_t *__restrict__ order, int64_t *__restrict__ n_inst, uint32_t *__restrict__ nbig,
            int32_t *__restrict__ status)
 {
@@ -647,9 +646,8 @@ k_scan_out(uint32_t *__restrict__ count, int64_t Ttot, int64_t capacity, const u
     }
 }
 
-__global__ void k_scatter(const float4 *__restrict__ rec, int64_t n, int V, Grid g,
-                          const uint32_t *__restrict__ start, uint32_t *__restrict__ cursor,
-                          uint64_t *__restrict__ keys, int64_t capacity)
+__global__ void k_scatter(const float4 *rec, int64_t n, int V, Grid g, const uint32_t *start,
+                          uint32_t *__restrict__ cursor, uint64_t *__restrict__ keys, int64_t capacity)
 {
     pdl_begin(rec, start, cursor, keys);
     const int64_t total = (int64_t)V * n;
@@ -675,8 +673,8 @@ __global__ void k_scatter(const float4 *__restrict__ rec, int64_t n, int V, Grid
 // instances per tile again, reserves one contiguous run per tile in each bucket with a
 // single global atomic, then places its instances with shared-memory atomics.
 __global__ void __launch_bounds__(kAggThreads, kAggMinBlocks)
-k_scatter_agg(const float4 *__restrict__ rec, int64_t n, int chunk, Grid g, const uint32_t *__restrict__ start,
-              uint32_t *__restrict__ cursor, const uint32_t *__restrict__ bcount, uint4 *__restrict__ slotrec,
+k_scatter_agg(const float4 *rec, int64_t n, int chunk, Grid g, const uint32_t *start,
+              uint32_t *__restrict__ cursor, const uint32_t *bcount, uint4 *__restrict__ slotrec,
               uint64_t *__restrict__ keys, int64_t capacity)
 {
     pdl_begin(rec, start, cursor, bcount, slotrec, keys);
@@ -912,7 +910,7 @@ __device__ __forceinline__ bool bucket_sort_tile(SortSmem<NTH, CAP> &sm, uint32_
 // Sort of one tile's list (2 <= len <= CAP keys) in shared memory by a block of NTH
 // threads, written to vals as slot ids: the bucket sort, else the stable LSD radix sort.
 template <int NTH, int CAP>
-__device__ __forceinline__ void sort_tile(SortSmem<NTH, CAP> &sm, const uint64_t *__restrict__ keys,
+__device__ __forceinline__ void sort_tile(SortSmem<NTH, CAP> &sm, const uint64_t *keys,
                                           uint32_t *__restrict__ vals, uint32_t st, uint32_t len)
 {
     constexpr int NW = NTH / 32;
@@ -1065,7 +1063,7 @@ static_assert(sizeof(SortSmem<kSortThreadsL, kSmallCap>) <= 48 * 1024, "static s
 
 // Tiles of at most kSortCapS keys; longer ones are listed (mid) for k_sort_tiles_l.
 __global__ void __launch_bounds__(kSortThreadsS)
-k_sort_tiles(const uint32_t *__restrict__ ranges, const uint64_t *__restrict__ keys, uint32_t *__restrict__ vals,
+k_sort_tiles(const uint32_t *ranges, const uint64_t *keys, uint32_t *__restrict__ vals,
              uint32_t *__restrict__ mid, uint32_t *__restrict__ nmid)
 {
     pdl_begin(ranges, keys, vals, mid, nmid);
@@ -1087,8 +1085,8 @@ k_sort_tiles(const uint32_t *__restrict__ ranges, const uint64_t *__restrict__ k
 
 // The listed longer tiles (persistent blocks); those above kSmallCap go to k_sort_big.
 __global__ void __launch_bounds__(kSortThreadsL)
-k_sort_tiles_l(const uint32_t *__restrict__ ranges, const uint64_t *__restrict__ keys, uint32_t *__restrict__ vals,
-               const uint32_t *__restrict__ mid, const uint32_t *__restrict__ nmid, uint32_t *__restrict__ big,
+k_sort_tiles_l(const uint32_t *ranges, const uint64_t *keys, uint32_t *__restrict__ vals,
+               const uint32_t *mid, const uint32_t *nmid, uint32_t *__restrict__ big,
                uint32_t *__restrict__ nbig)
 {
     pdl_begin(ranges, keys, vals, mid, nmid, big, nbig);
@@ -1107,8 +1105,8 @@ k_sort_tiles_l(const uint32_t *__restrict__ ranges, const uint64_t *__restrict__
 }
 
 __global__ void __launch_bounds__(kBigThreads)
-k_sort_big(const uint32_t *__restrict__ ranges, uint64_t *__restrict__ keys, uint32_t *__restrict__ vals,
-           const uint32_t *__restrict__ big, const uint32_t *__restrict__ nbig)
+k_sort_big(const uint32_t *ranges, uint64_t *__restrict__ keys, uint32_t *__restrict__ vals,
+           const uint32_t *big, const uint32_t *nbig)
 {
     pdl_begin(ranges, keys, vals, big, nbig);
     extern __shared__ uint64_t sbig[];

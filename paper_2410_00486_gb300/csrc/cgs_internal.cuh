@@ -38,10 +38,14 @@ __host__ __device__ inline Layout param_layout(int64_t n, int deg)
 // while its predecessor in the stream still drains, which hides its launch latency.  Every
 // such kernel begins with pdl_begin(): it lets its own successor be placed in turn, then waits
 // until everything before it in the stream is complete and visible (the predecessor itself
-// came back from this wait, so completion is transitive).  The kernel's pointers go through
-// pdl_begin() so that no read, not even one the compiler takes for a read of constant memory,
-// can be moved ahead of the wait.  Behind anything but such a kernel the launch is an
-// ordinary one.  The chain of an iteration uses it: four views' render 462 -> 440 us, three
+// came back from this wait, so completion is transitive).  What such a kernel reads may thus
+// be written while the kernel is already resident, and the non-coherent path (__ldg,
+// ld.global.nc) is defined only for memory that nothing writes during a kernel's whole
+// life: these kernels read through plain loads, which the wait orders, and take no
+// pointer to const as __restrict__, from which the compiler would form non-coherent loads.
+// The pointers go through pdl_begin() so that no read is moved ahead of the wait.  Behind
+// anything but such a kernel the launch is an ordinary one, and an ordinary launch behind
+// such a kernel waits for its end.  The chain of an iteration uses it: four views' render 462 -> 440 us, three
 // views with the SSIM loss 501 -> 478, one 640x480 view 212 -> 208, Adam's two kernels 105 ->
 // 100.  The loss of Eq. 9 and density control gained nothing from it (197 -> 222 and 119 -> 127
 // us, their loads no longer read-only ones) and are launched the ordinary way.

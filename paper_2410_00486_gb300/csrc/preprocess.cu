@@ -269,8 +269,8 @@ __device__ __forceinline__ void async_copy(float *dst, const float *src, bool wi
 // before their four stores left a block several memory latencies: with one view of 100k
 // Gaussians, where staging is most of the work, the projection takes 8.1 us after 16.1.
 template <int DEG>
-__device__ __forceinline__ Staged stage(float *sm, const float *__restrict__ P, int64_t n, int64_t g0,
-                                        int cnt, const cgs_camera *__restrict__ cams, int V)
+__device__ __forceinline__ Staged stage(float *sm, const float *P, int64_t n, int64_t g0, int cnt,
+                                        const cgs_camera *cams, int V)
 {
     constexpr int K = (DEG + 1) * (DEG + 1);
     const Layout L = param_layout(n, DEG);
@@ -297,7 +297,7 @@ __device__ __forceinline__ Staged stage(float *sm, const float *__restrict__ P, 
     cur += 6 * kGB;
     // cameras: 20 ABI floats + centre c = -R^T t
     const float *cf = reinterpret_cast<const float *>(cams);
-    for (int i = threadIdx.x; i < V * 20; i += blockDim.x) cur[(i / 20) * kCamF + (i % 20)] = __ldg(cf + i);
+    for (int i = threadIdx.x; i < V * 20; i += blockDim.x) cur[(i / 20) * kCamF + (i % 20)] = cf[i];
     asm volatile("cp.async.wait_all;" ::: "memory");
     __syncthreads();
     for (int v = threadIdx.x; v < V; v += blockDim.x) {
@@ -330,7 +330,7 @@ __host__ __device__ constexpr int staged_floats()
 
 template <int DEG>
 __global__ void __launch_bounds__(kPreThreads)
-k_preprocess(const float *__restrict__ P, int64_t n, const cgs_camera *__restrict__ cams, int V,
+k_preprocess(const float *P, int64_t n, const cgs_camera *cams, int V,
              Grid grid, float near_z, float4 *__restrict__ rec, float4 *__restrict__ sgrad)
 {
     pdl_begin(P, cams, rec, sgrad);
@@ -526,8 +526,8 @@ __device__ __forceinline__ void sigma_bwd(const Staged &st, int gl, const float 
 // view, by HBM.
 template <int DEG>
 __global__ void __launch_bounds__(kPreThreads, kPreBwdMinBlocks)
-k_preprocess_bwd(const float *__restrict__ P, int64_t n, const cgs_camera *__restrict__ cams, int V,
-                 Grid grid, float near_z, const float4 *__restrict__ rec, const float4 *__restrict__ sgrad,
+k_preprocess_bwd(const float *P, int64_t n, const cgs_camera *cams, int V,
+                 Grid grid, float near_z, const float4 *rec, const float4 *sgrad,
                  float *__restrict__ pgrad, int accumulate, float *__restrict__ accum,
                  float *__restrict__ denom, float *__restrict__ max_r2d)
 {
@@ -560,7 +560,7 @@ k_preprocess_bwd(const float *__restrict__ P, int64_t n, const cgs_camera *__res
             for (int k = 0; k < kViewChunk / 2; k++) {   // all loads in flight together
                 if (h0 + k >= V) break;
                 const float *r = reinterpret_cast<const float *>(rec + kRec4 * ((int64_t)(h0 + k) * n + slot0));
-                const int rad = __float_as_int(__ldg(r + 7));
+                const int rad = __float_as_int(r[7]);
                 if (rad > 0) vis |= 1u << k;
                 rmax = max(rmax, rad);
             }
@@ -574,16 +574,16 @@ k_preprocess_bwd(const float *__restrict__ P, int64_t n, const cgs_camera *__res
         const int64_t vstep = kRec4 * n;
         float4 G0 = make_float4(0.f, 0.f, 0.f, 0.f), G1 = G0;
         if (m) {
-            G0 = __ldg(gp + (__ffs(m) - 1) * vstep);
-            if (geometry) G1 = __ldg(gp + (__ffs(m) - 1) * vstep + 1);
+            G0 = gp[(__ffs(m) - 1) * vstep];
+            if (geometry) G1 = gp[(__ffs(m) - 1) * vstep + 1];
         }
         while (m) {
             const float *cam = st.cams + (v0 + __ffs(m) - 1) * kCamF;
             const float4 C0 = G0, C1 = G1;
             m &= m - 1u;
             if (m) {
-                G0 = __ldg(gp + (__ffs(m) - 1) * vstep);
-                if (geometry) G1 = __ldg(gp + (__ffs(m) - 1) * vstep + 1);
+                G0 = gp[(__ffs(m) - 1) * vstep];
+                if (geometry) G1 = gp[(__ffs(m) - 1) * vstep + 1];
             }
             if (geometry) {
                 Proj o;

@@ -158,11 +158,11 @@ __device__ __forceinline__ void bwd_item(const RasterBwdArgs &a, uint32_t place,
     auto fetch = [&](int at) {   // the lane's splat of the batch ending at `at`
         const int i = at - BD + lane;
         if (i >= 0) {
-            nslot = __ldg(a.vals + start + i);
+            nslot = a.vals[start + i];
             const float4 *r = a.rec + kRec4 * (size_t)nslot;
-            n0 = __ldg(r);
-            n1 = __ldg(r + 1);
-            n2 = __ldg(r + 2);
+            n0 = r[0];
+            n1 = r[1];
+            n2 = r[2];
         }
     };
     const int seg0 = SEG > 1 ? (int)((uint64_t)maxlast * seg / SEG) : 0;
@@ -185,10 +185,10 @@ __device__ __forceinline__ void bwd_item(const RasterBwdArgs &a, uint32_t place,
             for (int c0 = 0; c0 < BD; c0 += NT) {
                 const int i = c0 + tid;
                 if (i >= nraw) break;
-                const uint32_t slot = __ldg(a.vals + start + bstart + i);
+                const uint32_t slot = a.vals[start + bstart + i];
                 const float4 *r = a.rec + kRec4 * (size_t)slot;
-                const float4 r2 = __ldg(r + 2);
-                stage_splat(__ldg(r), __ldg(r + 1), r2.w, s0[i], s1[i]);
+                const float4 r2 = r[2];
+                stage_splat(r[0], r[1], r2.w, s0[i], s1[i]);
                 s2[i] = r2;
                 sslot[i] = slot;
             }
@@ -359,7 +359,7 @@ __device__ __forceinline__ void zero_rows(float (&red)[N], int t, int threads)
 template <int B, int BD>
 __global__ void __launch_bounds__(B *B / ppt_for<B, kPPTBwd>(), (min_blocks_for<B, kPPTBwd, kBwdMinWarps>())) k_render_bwd(RasterBwdArgs a)
 {
-    pdl_begin();   // the read-only loads below are addressed by what is read after the wait
+    pdl_begin();   // plain loads below: none moves ahead of the wait
     constexpr int PPT = ppt_for<B, kPPTBwd>();
     constexpr int NT = B * B / PPT;
     __shared__ BwdSmem<BD, NT * PPT, NT / 32> sm;
@@ -387,7 +387,7 @@ constexpr int kPartWarps = 4, kPartMinBlocks = 5;
 template <int S, int SEG>
 __global__ void __launch_bounds__(32 * kPartWarps, kPartMinBlocks) k_render_bwd_parts(RasterBwdArgs a)
 {
-    pdl_begin();   // the read-only loads below are addressed by what is read after the wait
+    pdl_begin();   // plain loads below: none moves ahead of the wait
     __shared__ BwdSmem<32, 256 / S, 1> smem[kPartWarps];
     auto &sm = smem[threadIdx.x >> 5];
     const int lane = threadIdx.x & 31;

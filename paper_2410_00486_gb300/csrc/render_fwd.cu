@@ -19,7 +19,7 @@ __device__ constexpr float kNoRow = __builtin_nanf("");
 template <int B, int BD, bool CKPT, bool COUNT, int PPT>
 __global__ void __launch_bounds__(B *B / PPT, (min_blocks_for<B, PPT, kFwdMinWarps>())) k_render_fwd(RasterFwdArgs a)
 {
-    pdl_begin();   // the read-only loads below are addressed by what is read after the wait
+    pdl_begin();   // plain loads below: none moves ahead of the wait
     constexpr int NT = B * B / PPT;
     constexpr int NW = NT / 32;
     __shared__ float4 s0[BD], s1[BD], s2[BD];
@@ -70,9 +70,9 @@ __global__ void __launch_bounds__(B *B / PPT, (min_blocks_for<B, PPT, kFwdMinWar
         const int cnt = (int)min((uint32_t)BD, end - base);
         for (int i = threadIdx.x; i < cnt; i += NT) {
             const uint32_t idx = base + (uint32_t)i;
-            const float4 *r = a.rec + kRec4 * (size_t)__ldg(a.vals + idx);
-            const float4 r2 = __ldg(r + 2);
-            stage_splat(__ldg(r), __ldg(r + 1), r2.w, s0[i], s1[i]);
+            const float4 *r = a.rec + kRec4 * (size_t)a.vals[idx];
+            const float4 r2 = r[2];
+            stage_splat(r[0], r[1], r2.w, s0[i], s1[i]);
             s2[i] = r2;
         }
         __syncthreads();
@@ -191,7 +191,7 @@ __global__ void __launch_bounds__(B *B / PPT, (min_blocks_for<B, PPT, kFwdMinWar
 // are pairs of floats until the last step (1200x680: 10.3 -> 5.1 us).
 constexpr int kLossThreads = 512;
 __global__ void __launch_bounds__(kLossThreads)
-k_loss_reduce(const float *__restrict__ partials, int64_t Tv, const float *__restrict__ weight, double inv3HW,
+k_loss_reduce(const float *partials, int64_t Tv, const float *weight, double inv3HW,
               float lambda_d, float *__restrict__ loss_view, int32_t *__restrict__ depth_count,
               int32_t *__restrict__ status)
 {
@@ -204,7 +204,7 @@ k_loss_reduce(const float *__restrict__ partials, int64_t Tv, const float *__res
 #pragma unroll 4
     for (int64_t t = threadIdx.x; t < Tv; t += kLossThreads)
 #pragma unroll
-        for (int k = 0; k < 3; k++) a[k].add(__ldg(p + kPartials * t + k));
+        for (int k = 0; k < 3; k++) a[k].add(p[kPartials * t + k]);
     auto warp_sum = [](PairSum x, int from) {
         for (int o = from; o > 0; o >>= 1) {
             PairSum y;
