@@ -371,7 +371,8 @@ int cgs_densify_apply(const float *params, const float *m, const float *v, int64
  * bytes, 256-byte aligned) holds a uniform grid of the points' bounding box (about one cell
  * per point of its volume, at most 128 cells per axis) and the points sorted by cell.
  * Outputs must not alias inputs.  A non-finite coordinate sets CGS_ERR_NONFINITE in
- * *status_dev (that point's outputs are then unspecified).
+ * *status_dev (that point's outputs are then unspecified, the others' distances are to the
+ * finite points; with fewer than min(3, n_points - 1) of those beside it, a point's d2 is 0).
  */
 size_t cgs_points_workspace(int64_t n_points);
 int cgs_points_to_gaussians(const float *params, const float *m, const float *v, int64_t n,

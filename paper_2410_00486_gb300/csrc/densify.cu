@@ -278,6 +278,7 @@ struct GridInfo {
     uint32_t box[6];   // sortable encodings, all maxima: complements of min x, y, z, then max x, y, z
     uint32_t done;     // blocks of k_bbox that have added their part
     uint32_t nfar;     // points listed for knn_far
+    uint32_t nbad;     // points with a coordinate that is not finite
     double sum[3], sumsq[3];
 };
 
@@ -355,13 +356,14 @@ k_bbox(const float *__restrict__ xyz, int64_t m, int64_t budget, GridInfo *__res
     __shared__ double smom[6][kBoxThreads];
     float lo[3] = {INFINITY, INFINITY, INFINITY}, hi[3] = {-INFINITY, -INFINITY, -INFINITY};
     double s1[3] = {0.0, 0.0, 0.0}, s2[3] = {0.0, 0.0, 0.0};
-    bool bad = false;
+    int bad = 0;
 #pragma unroll 4
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < m; i += (int64_t)gridDim.x * blockDim.x)
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < m; i += (int64_t)gridDim.x * blockDim.x) {
+        bool finite = true;
         for (int a = 0; a < 3; a++) {
             const float x = xyz[3 * i + a];
             if (!isfinite(x)) {
-                bad = true;
+                finite = false;
                 continue;
             }
             lo[a] = fminf(lo[a], x);
@@ -369,6 +371,8 @@ k_bbox(const float *__restrict__ xyz, int64_t m, int64_t budget, GridInfo *__res
             s1[a] += x;
             s2[a] += (double)x * x;
         }
+        bad += finite ? 0 : 1;
+    }
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     for (int a = 0; a < 3; a++) {
         for (int o = 16; o > 0; o >>= 1) {
@@ -383,7 +387,11 @@ k_bbox(const float *__restrict__ xyz, int64_t m, int64_t budget, GridInfo *__res
             sbox[w][3 + a] = any ? f2sortable(hi[a]) : 0u;
         }
     }
-    if (__any_sync(kFull, bad) && lane == 0) set_status(status, CGS_ERR_NONFINITE);
+    bad = __reduce_add_sync(kFull, bad);
+    if (bad > 0 && lane == 0) {
+        atomicAdd(&gi->nbad, (uint32_t)bad);
+        set_status(status, CGS_ERR_NONFINITE);
+    }
     __syncthreads();
     // one warp per sum: FP64 is slow on this part, a shuffle tree in every warp took most of
     // the kernel
@@ -457,11 +465,14 @@ struct Query {
     uint32_t self;     // position in cell order
     float p[3];
     int c[3];
-    int want;          // neighbours there are to find: min(3, points - 1)
+    // neighbours to find: min(3, points - 1); none if fewer of the others are finite, when the
+    // scale takes its floor (a missing neighbour's distance would be infinite)
+    int want;
 
     __device__ __forceinline__ Query(const GridInfo &gi, const float4 &q, uint32_t at, int64_t m)
         : g(gi), self(at), p{q.x, q.y, q.z}, want(m - 1 < kKnn ? (int)(m - 1) : kKnn)
     {
+        if (m - 1 - (int64_t)g.nbad < want) want = 0;
         for (int a = 0; a < 3; a++) c[a] = cell_axis(p[a], g.lo[a], g.h, g.G[a]);
     }
     __device__ __forceinline__ float dist2(const float4 &q) const
