@@ -8,6 +8,8 @@
 // -tau, both scaled by log2 e) before any exponential.  A block-wide vote
 // (__syncthreads_count) ends the walk as soon as every pixel of the tile is saturated (T below
 // 1e-4).
+#include <cooperative_groups.h>
+
 #include "raster.cuh"
 
 namespace cgs {
@@ -187,46 +189,63 @@ __global__ void __launch_bounds__(B *B / PPT, (min_blocks_for<B, PPT, kFwdMinWar
 
 // Per-view loss from the per-tile partial sums, summed in a fixed order (deterministic):
 //   L_v = w_v (sum|r_rgb| / (3 H W) + lambda_d sum|r_d| / count)   (count = valid depth pixels)
-// One block per view: FP64 sums, at two lanes a clock, took most of its time, so the sums
-// are pairs of floats until the last step (1200x680: 10.3 -> 5.1 us).
-constexpr int kLossThreads = 512;
-__global__ void __launch_bounds__(kLossThreads)
+// The sums are in FP64, whose adds and conversions an SM runs at two lanes a clock, so a view
+// of many tiles is summed by a cluster of C blocks on as many SMs.  Bound by that rate and,
+// below a thousand tiles, by latency.  Forward and this reduction with empty lists, one block
+// and eight (us): one view of 80 tiles 4.2, 5.0; of 512 6.1, 6.3; of 1200 9.4, 8.5; of 3225
+// 15.3, 11.3 (four blocks 11.5); 16 views of 3225 145, 136; one of 47000 245, 138.  Sums as
+// pairs of floats took 3.8, 5.3, 7.4, 10.0, 135 and 148, but held 45 bits and ended at float's
+// range, where a view's sum of large residuals became infinite though its mean was not.
+constexpr int kLossThreads = 128, kLossWarps = kLossThreads / 32;
+struct LossSums {
+    double rgb, depth;
+    unsigned long long count;
+    __device__ __forceinline__ void add(const LossSums &o)
+    {
+        rgb += o.rgb;
+        depth += o.depth;
+        count += o.count;
+    }
+};
+__device__ __forceinline__ LossSums warp_sum(LossSums x, int from)
+{
+    for (int o = from; o > 0; o >>= 1)
+        x.add(LossSums{__shfl_xor_sync(kFull, x.rgb, o), __shfl_xor_sync(kFull, x.depth, o),
+                       __shfl_xor_sync(kFull, x.count, o)});
+    return x;
+}
+
+template <int C>
+__global__ void __cluster_dims__(C, 1, 1) __launch_bounds__(kLossThreads)
 k_loss_reduce(const float *partials, int64_t Tv, const float *weight, double inv3HW,
               float lambda_d, float *__restrict__ loss_view, int32_t *__restrict__ depth_count,
               int32_t *__restrict__ status)
 {
     pdl_begin(partials, weight, loss_view, depth_count, status);
-    constexpr int NW = kLossThreads / 32;
-    __shared__ PairSum sh[3][NW];
-    const int v = blockIdx.x, lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    PairSum a[3];
+    static_assert(C <= 32 && (C & (C - 1)) == 0 && (kLossWarps & (kLossWarps - 1)) == 0, "a warp adds the last sums");
+    __shared__ LossSums sh[kLossWarps], own;
+    const int v = blockIdx.x / C, rank = blockIdx.x % C, lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    LossSums a{0.0, 0.0, 0ull};
     const float *p = partials + kPartials * (int64_t)v * Tv;
 #pragma unroll 4
-    for (int64_t t = threadIdx.x; t < Tv; t += kLossThreads)
-#pragma unroll
-        for (int k = 0; k < 3; k++) a[k].add(p[kPartials * t + k]);
-    auto warp_sum = [](PairSum x, int from) {
-        for (int o = from; o > 0; o >>= 1) {
-            PairSum y;
-            y.h = __shfl_xor_sync(kFull, x.h, o);
-            y.l = __shfl_xor_sync(kFull, x.l, o);
-            x.add(y);
-        }
-        return x;
-    };
-#pragma unroll
-    for (int k = 0; k < 3; k++) {
-        a[k] = warp_sum(a[k], 16);
-        if (lane == 0) sh[k][w] = a[k];
-    }
+    for (int64_t t = rank * kLossThreads + (int)threadIdx.x; t < Tv; t += C * kLossThreads)
+        a.add(LossSums{p[kPartials * t], p[kPartials * t + 1], (unsigned long long)p[kPartials * t + 2]});
+    a = warp_sum(a, 16);
+    if (lane == 0) sh[w] = a;
     __syncthreads();
-    if (w > 0) return;
-#pragma unroll
-    for (int k = 0; k < 3; k++) a[k] = warp_sum(sh[k][lane % NW], NW / 2);
-    if (lane == 0) {
+    if (w == 0) a = warp_sum(sh[lane % kLossWarps], kLossWarps / 2);
+    if constexpr (C > 1) {
+        namespace cg = cooperative_groups;
+        cg::cluster_group cluster = cg::this_cluster();
+        if (threadIdx.x == 0) own = a;
+        cluster.sync();   // every block's sums are there
+        if (rank == 0 && w == 0) a = warp_sum(*cluster.map_shared_rank(&own, lane % C), C / 2);
+        cluster.sync();   // and have been read
+    }
+    if (rank == 0 && threadIdx.x == 0) {
         const double wv = weight ? (double)weight[v] : 1.0;
-        const double cnt = a[2].value();
-        const double L = wv * (a[0].value() * inv3HW + (cnt > 0.0 ? (double)lambda_d * a[1].value() / cnt : 0.0));
+        const double cnt = (double)a.count;
+        const double L = wv * (a.rgb * inv3HW + (cnt > 0.0 ? (double)lambda_d * a.depth / cnt : 0.0));
         loss_view[v] = (float)L;
         depth_count[v] = (int32_t)cnt;
         if (!isfinite(L)) set_status(status, CGS_ERR_NONFINITE);
@@ -281,12 +300,19 @@ cudaError_t raster_fwd(const RasterFwdArgs &a, int B, int BD, cudaStream_t s)
     }
 }
 
+constexpr int kLossCluster = 8;               // blocks a view
+constexpr int64_t kLossClusterTiles = 512;    // up to this many tiles in a view one block is as fast
+
 cudaError_t loss_reduce(const float *partials, const Grid &g, int V, const float *weight, float lambda_d,
                         float *loss_view, int32_t *depth_count, int32_t *status, cudaStream_t s)
 {
     const double inv3HW = 1.0 / (3.0 * (double)g.W * (double)g.H);
-    launch(k_loss_reduce, V, kLossThreads, 0, s, partials, g.Tv, weight, inv3HW, lambda_d, loss_view, depth_count,
-           status);
+    if (g.Tv > kLossClusterTiles)
+        launch(k_loss_reduce<kLossCluster>, V * kLossCluster, kLossThreads, 0, s, partials, g.Tv, weight, inv3HW,
+               lambda_d, loss_view, depth_count, status);
+    else
+        launch(k_loss_reduce<1>, V, kLossThreads, 0, s, partials, g.Tv, weight, inv3HW, lambda_d, loss_view,
+               depth_count, status);
     return cudaGetLastError();
 }
 
