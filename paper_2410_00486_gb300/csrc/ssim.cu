@@ -24,6 +24,7 @@ constexpr int kSsimIn = kSsimT + 2 * kSsimR;  // staged edge
 constexpr float kC1 = 0.0001f, kC2 = 0.0009f;
 constexpr int kRB = 4;                       // outputs per thread along a blur pass
 constexpr int kSsimThreads = kSsimT * kSsimT / kRB;
+constexpr int kSsimMaxSteps = 8;       // steps of a strip at most
 constexpr int kSsimMinBlocks = 3000;   // blocks a window should have before its strips get longer
 static_assert(kSsimT * (kSsimT / kRB) == kSsimThreads, "a pass over a tile is one round of the block");
 
@@ -354,10 +355,11 @@ k_ssim_bwd(const float *__restrict__ img, const float *__restrict__ tgt, const f
                 dl_ddepth[pix] = gd;
             }
         }
-        sD.add(absd);
+        // (scaled so that a warp's sum over a strip leaves float's range no sooner than one over a tile)
+        sD.add(absd * (1.f / kSsimMaxSteps));
     }
     if (ch == 0) {
-        const double s = block_total(sD, red);
+        const double s = kSsimMaxSteps * block_total(sD, red);
         if (threadIdx.x == 0) atomicAdd(acc + kSsimAcc * v + 2, s);
     }
     if (threadIdx.x == 0) {
@@ -386,7 +388,7 @@ static int ssim_steps(int W, int H, int V)
 {
     const int64_t cols = (W + kSsimT - 1) / kSsimT, rows = (H + kSsimT - 1) / kSsimT;
     int steps = 1;
-    while (steps < 8 && cols * ((rows + steps) / (steps + 1)) * 3 * V >= kSsimMinBlocks) steps++;
+    while (steps < kSsimMaxSteps && cols * ((rows + steps) / (steps + 1)) * 3 * V >= kSsimMinBlocks) steps++;
     return steps;
 }
 
