@@ -113,12 +113,20 @@ static int64_t chunk_count_entries(int64_t n, int64_t V, int64_t Tv, int chunk)
     return (n + chunk - 1) / chunk * V * Tv;
 }
 
-// Bytes for every chunk size that n or fewer Gaussians may take: chunks below kChunkSmall come
-// to at most 2 num_sms blocks, so a workspace kept for a growing map also serves a smaller one.
+// Bytes for every chunk size that n or fewer Gaussians may take, so a workspace kept for a
+// growing map also serves a smaller one.  A smaller map may take smaller chunks and need more
+// block counts: chunks of 1024 while ceil(n / 2048) V < 4 num_sms, chunks below that while
+// their blocks are fewer than 2 num_sms.
 size_t bin_ws_bytes(int64_t capacity, int64_t n, int64_t V, int64_t Tv, int num_sms)
 {
     int64_t counts = chunk_count_entries(n, V, Tv, chunk_for(n, V, num_sms));
-    if (counts > 0) counts = std::max(counts, std::min((n + kChunkMin - 1) / kChunkMin * V, 2 * (int64_t)num_sms) * Tv);
+    if (counts > 0) {
+        auto chunks = [&](int chunk) { return (n + chunk - 1) / chunk; };
+        constexpr int kHalves = kChunkLarge / kChunkSmall;
+        const int64_t small = std::min(chunks(kChunkSmall), kHalves * ((4 * (int64_t)num_sms - 1) / V)) * V;
+        const int64_t fine = std::min(chunks(kChunkMin) * V, 2 * (int64_t)num_sms);
+        counts = std::max({counts, small * Tv, fine * Tv});
+    }
     return ws_layout(capacity, Tv * V, counts, V * n, nullptr, nullptr);
 }
 
