@@ -82,7 +82,8 @@ typedef struct {
     float bg[3];             /* background colour added with the final transmittance */
     float lambda_depth;      /* weight of the masked depth L1 term (0.1) */
     int32_t batch_depth_bwd; /* splats per batch in the pixel-wise raster backward: 0 (same as
-                                batch_depth), 32, 64, 128 or 256 */
+                                batch_depth), 32, 64, 128 or 256; windows of few 16x16 tiles
+                                take 32 whatever it says (cgs_raster_bwd_batch) */
     int32_t count_work;      /* nonzero: cgs_render_fwd also counts the (splat, pixel) pairs it
                                 blends (per-tile partial 4; a per-pair counter, about 5% of the
                                 blend's time); 0: that partial is written as 0 */
@@ -239,6 +240,11 @@ int cgs_raster_bwd(const float *rec, const uint32_t *vals, const uint32_t *range
                    const float *tgt_depth, const int32_t *depth_count, const float *dl_dimg,
                    const float *dl_ddepth, float *slot_grad, uint32_t *work, int32_t *status_dev,
                    void *stream);
+
+/* Splats per batch that cgs_raster_bwd takes for V views on the current device: the batch
+ * depth asked for, or 32 where it divides 16x16 tiles among warps, one splat a lane (windows
+ * of at most 32 tiles per multiprocessor).  Sizes only: results do not depend on it. */
+int32_t cgs_raster_bwd_batch(int32_t V, const cgs_config *cfg);
 
 /*
  * Splat-wise backward (Sec. III-C.1 and Fig. 4a: the paper's backward).  The forward

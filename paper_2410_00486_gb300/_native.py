@@ -73,6 +73,7 @@ _SIGS = {
                                        _P, c_int64, _P, _P, _P, _P]),
     "cgs_raster_bwd": (c_int32, [_P, _P, _P, _P, c_int32, _P, _P, _P, _P, _P, _P, _P, _P, _P, _P, _P,
                                  _P, _P, _P, _P]),
+    "cgs_raster_bwd_batch": (c_int32, [c_int32, _P]),
     "cgs_preprocess_bwd": (c_int32, [_P, c_int64, _P, c_int32, _P, _P, _P, _P, c_int32, _P, _P, _P,
                                      _P, _P]),
     "cgs_render_bwd": (c_int32, [_P, c_int64, _P, c_int32, _P, _P, _P, _P, _P, _P, _P, _P, _P, _P, _P,
@@ -237,6 +238,10 @@ def cgs_raster_bwd(rec, vals, ranges, tile_order, V, cfg, view_weight, img, dept
         _dev(rec), _dev(vals), _dev(ranges), _dev(tile_order), V, byref(cfg), _dev(view_weight), _dev(img),
         _dev(depth), _dev(t_final), _dev(last), _dev(tgt_rgb), _dev(tgt_depth), _dev(depth_count),
         _dev(dl_dimg), _dev(dl_ddepth), _dev(slot_grad), _dev(work), _dev(status), _stream(stream)))
+
+
+def cgs_raster_bwd_batch(V, cfg) -> int:
+    return lib().cgs_raster_bwd_batch(V, byref(cfg))
 
 
 def cgs_preprocess_bwd(params, n, cams, V, cfg, rec, slot_grad, param_grad, accumulate=False, accum=None,

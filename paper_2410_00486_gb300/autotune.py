@@ -3,7 +3,8 @@
 candidate runs the whole captured window iteration on the caller's scene; the fastest
 (CUDA-event time) wins.  First every (tile, depth) pair with one depth for both kernels,
 then, at the best tile, each kernel's depth on its own (the two kernels are separate
-launches, so their best depths are independent).  Results are cached per workload shape
+launches, so their best depths are independent).  A backward depth that the window does not
+take (cgs_raster_bwd_batch) is not a candidate.  Results are cached per workload shape
 in memory and, when `cache_path` is given, in a JSON file.
 """
 from __future__ import annotations
@@ -13,6 +14,7 @@ from pathlib import Path
 
 import torch
 
+from . import _native as N
 from .window import MappingWindow
 
 CANDIDATES = [(t, bd) for t in (8, 16, 32) for bd in (32, 64, 128, 256)]
@@ -51,6 +53,9 @@ def autotune(params: torch.Tensor, n: int, sh_degree: int, width: int, height: i
         return _memo[key]
     results = {}
 
+    def bwd_depth(tile, bd):               # the depth the backward takes when asked for bd
+        return N.cgs_raster_bwd_batch(views, N.make_config(width, height, tile, bd, sh_degree))
+
     def measure(tile, bd, bdb):
         if (tile, bd, bdb) in results:
             return
@@ -68,14 +73,14 @@ def autotune(params: torch.Tensor, n: int, sh_degree: int, width: int, height: i
         torch.cuda.empty_cache()
 
     for tile, bd in candidates:
-        measure(tile, bd, bd)
+        measure(tile, bd, bwd_depth(tile, bd))
     tile, bd, bdb = min(results, key=results.get)
     depths = sorted({b for _, b in candidates})
     for d in depths:                       # forward depth, backward depth held
         measure(tile, d, bdb)
     bd = min((d for d in depths), key=lambda d: results[(tile, d, bdb)])
     for d in depths:                       # backward depth, forward depth held
-        measure(tile, bd, d)
+        measure(tile, bd, bwd_depth(tile, d))
     best = min(results, key=results.get)
     _memo[key] = (best, results)
     if cache_path:

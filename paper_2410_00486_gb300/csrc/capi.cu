@@ -193,6 +193,13 @@ int cgs_raster_bwd(const float *rec, const uint32_t *vals, const uint32_t *range
     return cuda_status(raster_bwd(a, cfg->tile, bd, num_sms(), (cudaStream_t)stream));
 }
 
+int32_t cgs_raster_bwd_batch(int32_t V, const cgs_config *cfg)
+{
+    if (V < 1 || V > kMaxViews || !cfg_ok(cfg)) return CGS_ERR_ARG;
+    const int bd = cfg->batch_depth_bwd ? cfg->batch_depth_bwd : cfg->batch_depth;
+    return raster_bwd_batch(make_grid(*cfg).Tv * V, cfg->tile, bd, num_sms());
+}
+
 int cgs_preprocess_bwd(const float *params, int64_t n, const cgs_camera *cams, int32_t V, const cgs_config *cfg,
                        const float *rec, const float *slot_grad, float *param_grad, int32_t accumulate, float *accum,
                        float *denom, float *max_r2d, int32_t *status_dev, void *stream)

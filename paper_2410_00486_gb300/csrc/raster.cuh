@@ -168,5 +168,7 @@ __device__ __forceinline__ float staged_power(const float4 &t0, float hC, float 
 int num_sms();
 cudaError_t raster_fwd(const RasterFwdArgs &a, int B, int BD, cudaStream_t s);
 cudaError_t raster_bwd(const RasterBwdArgs &a, int B, int BD, int sms, cudaStream_t s);
+// Splats per batch that raster_bwd takes for a window of so many tiles.
+int raster_bwd_batch(int64_t tiles, int B, int BD, int sms);
 
 }  // namespace cgs

@@ -383,12 +383,12 @@ __global__ void __launch_bounds__(B *B / ppt_for<B, kPPTBwd>(), (min_blocks_for<
 
 // Windows of few 16x16 tiles (bwd_split): the warps of a block of four take parts of tiles,
 // each on its own.
-constexpr int kPartWarps = 4, kPartMinBlocks = 5;
+constexpr int kPartWarps = 4, kPartMinBlocks = 5, kPartBatch = 32;   // a splat of a batch per lane
 template <int S, int SEG>
 __global__ void __launch_bounds__(32 * kPartWarps, kPartMinBlocks) k_render_bwd_parts(RasterBwdArgs a)
 {
     pdl_begin();   // plain loads below: none moves ahead of the wait
-    __shared__ BwdSmem<32, 256 / S, 1> smem[kPartWarps];
+    __shared__ BwdSmem<kPartBatch, 256 / S, 1> smem[kPartWarps];
     auto &sm = smem[threadIdx.x >> 5];
     const int lane = threadIdx.x & 31;
     zero_rows(sm.red, lane, 32);
@@ -403,7 +403,8 @@ __global__ void __launch_bounds__(32 * kPartWarps, kPartMinBlocks) k_render_bwd_
             break;
         }
         if (item >= n_items) break;
-        bwd_item<16, 32, 32, 8 / S, S, SEG>(a, item / (S * SEG), (int)(item / SEG % S), (int)(item % SEG), lane, sm);
+        bwd_item<16, kPartBatch, 32, 8 / S, S, SEG>(a, item / (S * SEG), (int)(item / SEG % S), (int)(item % SEG), lane,
+                                                    sm);
     }
 }
 
@@ -426,6 +427,11 @@ static BwdSplit bwd_split(int64_t tiles, int sms)
     if (tiles <= 8 * (int64_t)sms) return BwdSplit{4, 2};
     if (tiles <= 16 * (int64_t)sms) return BwdSplit{4, 1};
     return BwdSplit{tiles <= 32 * (int64_t)sms ? 2 : 1, 1};
+}
+
+int raster_bwd_batch(int64_t tiles, int B, int BD, int sms)
+{
+    return B == 16 && bwd_split(tiles, sms).parts > 1 ? kPartBatch : BD;
 }
 
 // Blocks of a persistent launch: as many as are resident on the GPU (queried once per device
