@@ -62,12 +62,12 @@ __device__ __forceinline__ void pdl_begin(T &...pointers)
     (after_wait(pointers), ...);
 }
 
-template <class... K, class... A>
+template <bool DEPENDENT = true, class... K, class... A>
 inline cudaError_t launch(void (*kernel)(K...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, A &&...args)
 {
     cudaLaunchAttribute attr = {};
     attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr.val.programmaticStreamSerializationAllowed = 1;
+    attr.val.programmaticStreamSerializationAllowed = DEPENDENT;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid;
     cfg.blockDim = block;

@@ -464,7 +464,12 @@ static cudaError_t launch_bwd(const RasterBwdArgs &a, int sms, cudaStream_t s)
         const cudaError_t e = persistent_blocks(a, k_render_bwd<B, BD>, nt, resident, sms, blocks, s);
         if (e != cudaSuccess) return e;
     }
-    if (blocks > 0) launch(k_render_bwd<B, BD>, (unsigned)blocks, nt, 0, s, a);
+    // Not a dependent launch: placed beside its predecessor's last blocks, a grid of few large
+    // blocks lies unevenly on the SMs and the longest lists share one.  Forward to parameter
+    // gradients, placed early and not (us): one 640x480 view of 46k in 32x32 tiles 488, 448
+    // (184k: 773, 709); 800x600 of 72k 589, 562; eight of 46k in 16x16 tiles 679, 656; one in
+    // 8x8 tiles 248, 222; four 1200x680 views of 122k 1244 both.
+    if (blocks > 0) launch<false>(k_render_bwd<B, BD>, (unsigned)blocks, nt, 0, s, a);
     return cudaGetLastError();
 }
 
