@@ -77,7 +77,7 @@ struct BinWs {
 
 static inline size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 
-// Sections: counters (one memset), big-tile list, per-chunk counts and per-slot bin
+// Sections: counters (set by one kernel), big-tile list, per-chunk counts and per-slot bin
 // records (shared-memory path only), keys.
 static size_t ws_layout(int64_t capacity, int64_t Ttot, int64_t chunk_counts, int64_t slots, BinWs *w, void *base)
 {
@@ -677,9 +677,9 @@ __global__ void k_scatter(const float4 *rec, int64_t n, int V, Grid g, const uin
     }
 }
 
-// Aggregated scatter (same block decomposition as k_count_agg): the block counts its
-// instances per tile again, reserves one contiguous run per tile in each bucket with a
-// single global atomic, then places its instances with shared-memory atomics.
+// Aggregated scatter (same block decomposition as k_count_agg): the block reads the count
+// pass's counts of its instances per tile, reserves one contiguous run per tile in each bucket
+// with a single global atomic, then places its instances with shared-memory atomics.
 __global__ void __launch_bounds__(kAggThreads, kAggMinBlocks)
 k_scatter_agg(const float4 *rec, int64_t n, int chunk, Grid g, const uint32_t *start,
               uint32_t *__restrict__ cursor, const uint32_t *bcount, uint4 *__restrict__ slotrec,

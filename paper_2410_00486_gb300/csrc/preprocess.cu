@@ -15,7 +15,8 @@ namespace cgs {
 constexpr int kGB = 128;         // Gaussians per block (64: backward 0.53 ms, 128: 0.44 on the 16-view window)
 constexpr int kPreThreads = 256;
 // Resident blocks per SM the backward is compiled for (at most 85 registers, 61 KB of shared
-// memory on 16 views).
+// memory on 16 views).  At the 80 registers that leaves a thread spills 112 bytes at SH degree
+// 3, 120 at degree 2.
 constexpr int kPreBwdMinBlocks = 3;
 constexpr int kViewChunk = 32;   // views whose visibility the backward holds at a time (one word a Gaussian)
 static_assert(kPreThreads == 2 * kGB, "the backward gives a Gaussian two threads");

@@ -64,9 +64,9 @@ __device__ __forceinline__ void item_tile(const uint32_t *order, const Grid &g, 
 // the staged splat is read from shared memory once for PPT pixels and the backward's
 // per-(warp, splat) reduction covers 32*PPT pixels.
 // The forward keeps two (its per-thread state is small and occupancy pays; four measured
-// slower; one on windows of few tiles), the backward eight: one warp per 16x16 tile, half the warp reductions per pixel
-// of four pixels, which were a third of its time (3.84 vs 4.04 ms on the 16-view window);
-// on windows of few tiles four or two, a part of the tile per warp.
+// slower; one on windows of few tiles), the backward eight: one warp per 16x16 tile, half the
+// warp reductions per pixel of four pixels, which were a third of its time (3.84 vs 4.04 ms on
+// the 16-view window); on windows of few tiles four or two, a part of the tile per warp.
 constexpr int kPPTFwd = 2;
 constexpr int kPPTBwd = 8;
 

@@ -419,6 +419,7 @@ __global__ void __launch_bounds__(32 * kPartWarps, kPartMinBlocks) k_render_bwd_
 // 173; 3225 tiles 307, 276, 333; 3600 tiles 365, 275, 325; 5700 tiles 464, 521, 632; 9600 tiles
 // 767, 833, 966.  Two parts in two segments: 158 at 1900 tiles, 106 at 2394, else slower.
 // Splitting only the longest lists' tiles: 3225 tiles 314 to 395, 5700 tiles 493 to 602.
+// The lines lie between measured sizes: 1200 and 1900 tiles, 2394 and 3225, 3600 and 5700.
 struct BwdSplit {
     int parts, segments;
 };

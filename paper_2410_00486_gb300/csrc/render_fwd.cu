@@ -257,6 +257,7 @@ k_loss_reduce(const float *partials, int64_t Tv, const float *weight, double inv
 // a larger one by the issue of all its steps.  Measured (us, two pixels and one): 80 tiles
 // 15.6, 15.2; 300 tiles 17.8, 15.1; 475 tiles 22.1, 20.5; 1200 tiles 46.7, 35.5 (longer lists
 // 81, 62); 1900 tiles 53, 56; 2394 tiles 33, 39; 3600 tiles 92, 110; 9600 tiles 252, 298.
+// Nothing between 1200 and 1900 tiles was measured both ways; the line lies just above 1200.
 constexpr int kFwdWideTiles = 8;
 
 template <int B, int BD>
